@@ -224,7 +224,7 @@ def kernel_sources_sha256():
     import hashlib
     import re
     h = hashlib.sha256()
-    for f in ("kn_integrate.cu", "kn_internal.h", "kn_tables.cu"):
+    for f in ("kn_integrate.cu", "kn_slots.cu", "kn_device.cuh", "kn_internal.h", "kn_tables.cu"):
         txt = open(os.path.join(ROOT, "paper_1409_5826_gb300", "csrc", f)).read()
         txt = re.sub(r"/\*.*?\*/", "", txt, flags=re.S)
         txt = re.sub(r"//[^\n]*", "", txt)

@@ -145,7 +145,12 @@ typedef struct {
        threads_per_cta is CTA-per-zone.  The built-in default for one network
        stages the tables in shared memory and takes, in KN_PREC_MIXED with
        groups of more than one warp, up to 5 groups per CTA and then the largest
-       group; otherwise the most groups per CTA and then the smallest group. */
+       group; otherwise the most groups per CTA and then the smallest group.
+       In KN_PREC_MIXED kn_integrate_batch (without replay, mlp or records) takes
+       from the tiling only the order of its sums, which threads_per_zone sets: how
+       many zones and threads share an SM then follows from the zone count, with the
+       same results bit for bit.  Networks beyond that kernel's capacities run as
+       tiled. */
     int32_t threads_per_cta;
     int32_t threads_per_zone;
     int32_t use_graph;     /* 1: capture the launch sequence in a CUDA graph and replay it */
@@ -269,7 +274,8 @@ kn_status kn_network_info(const kn_network *net, int32_t *n_species, int32_t *n_
  * (a multiple of 32 in [32, 1024]); no device is touched.  The F+ and k sums
  * of Eq. 1 (Sec. 10 item (2)) are laid out as warp slices of row pieces; the
  * builder verifies every index and destination and, running the gather on
- * the host with V[v] = v + 1, that every row's sum comes out exactly once.
+ * the host with V[v] = v + 1, that every row's sum comes out exactly once
+ * (KN_PREC_MIXED: through every table that kn_integrate_batch may use).
  * stats (4 int32, caller-owned) receives: the piece length cap L, the number
  * of slices, the longest warp's terms per lane, and the table bytes.
  * Errors: KN_ERR_INVALID_ARG (as kn_create_network, or a bad precision or

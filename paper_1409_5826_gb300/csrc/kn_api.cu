@@ -123,6 +123,7 @@ static kn_status device_info(DeviceInfo& d) {
     }
     if (!g_smem_limit_set) {
         KN_CUDA(integrator_set_smem_limit(g_dev.smem_optin - 1024));
+        KN_CUDA(slots_set_smem_limit(g_dev.smem_optin - 1024));
         g_smem_limit_set = 1;
     }
     d = g_dev;
@@ -171,6 +172,88 @@ static kn_status plan_tiling(kn_network* n, int prec, int P, int budget, int G_f
     if (have) {
         out = best;
         ok = true;
+    }
+    return KN_OK;
+}
+
+// The slot tables of one network for (G, T, NZ, cap), built on first use.
+static kn_status get_slots(kn_network* n, int G, int T, int NZ, int cap, SlotBlob** out) {
+    Tables& tb = n->tables.at({kPrecMixed, G});
+    auto it = tb.slots.find({T, NZ});
+    if (it == tb.slots.end()) {
+        std::vector<unsigned char> blob;
+        SlotBlob sb;
+        kn_status s = build_slots_host(n, tb, T, NZ, cap, blob, sb.st, sb.fits);
+        if (s != KN_OK) return s;
+        if (sb.fits) {
+            sb.blob.reset(new DevBuf());
+            KN_CUDA(sb.blob->ensure(blob.size()));
+            KN_CUDA(cudaMemcpy(sb.blob->p, blob.data(), blob.size(), cudaMemcpyHostToDevice));
+        }
+        it = tb.slots.emplace(std::make_pair(T, NZ), std::move(sb)).first;
+    }
+    *out = &it->second;
+    return KN_OK;
+}
+
+// Plan the several-zones-per-group kernel (kn_slots.cu) for networks whose
+// summation orders are those of group sizes tl[p].G: zones per group, threads
+// per group and groups per CTA.  ok = false: the group kernel runs.
+static kn_status plan_slots(kn_network* const* nets, int n_nets, const Tiling* tl, int sms, int budget, bool qss,
+                            LaunchParams& lp, int& grid, int& block, bool& ok) {
+    ok = false;
+    int zones = 0;
+    for (int p = 0; p < n_nets; ++p) {
+        if (tl[p].G < nets[p]->N) return KN_OK;
+        zones += lp.plans[p].n_zones;
+    }
+    // Zones per SM.  Two zones to a group where an SM gets three or more: a pair's
+    // step takes less than twice a single zone's (150/1604, 256 threads: 2.3 against
+    // 1.5 us an attempt), and up to two zones, one to a group, finish sooner.
+    const int zps = (zones + sms - 1) / sms;
+    for (int NZ = zps > 2 ? 2 : 1; NZ >= 1; --NZ) {
+        bool all = true;
+        int bytes = 0, threads = 0;
+        for (int p = 0; p < n_nets && all; ++p) {
+            kn_network* n = nets[p];
+            PlanDev& P = lp.plans[p];
+            const bool warp = tl[p].G == 32;
+            if (warp && !rate_cache_on(n, kPrecMixed)) return KN_OK;
+            const int cap = warp ? kCapWarp : (rate_cache_on(n, kPrecMixed) ? kCapGroup : kCapEvery);
+            // the most groups that the zones can use, each of at least the species'
+            // warps and the one that decides, then all threads to those groups
+            const int lo = warp ? 32 : (n->N + 31) / 32 * 32 + 32;
+            int ng = std::min(warp ? kSlotThreads / 32 : kMaxGroups, kSlotThreads / lo);
+            ng = std::max(1, std::min(ng, (zps + NZ - 1) / NZ));
+            bool fit = false;
+            for (; ng >= 1 && !fit; --ng) {
+                const int T = warp ? 32 : kSlotThreads / ng / 32 * 32;
+                if (T < lo) continue;
+                SlotBlob* sb;
+                kn_status s = get_slots(n, tl[p].G, T, NZ, cap, &sb);
+                if (s != KN_OK) return s;
+                if (!sb->fits) continue;
+                const SlotLayout sl = slot_layout(n, sb->st, T, NZ, qss);
+                if (sb->st.bytes + ng * sl.bytes > budget) continue;
+                P.slot_blob = (const unsigned char*)sb->blob->p;
+                P.st = sb->st;
+                P.sl = sl;
+                P.T = T;
+                P.ng = ng;
+                P.cap = cap;
+                fit = true;
+                bytes = std::max(bytes, P.st.bytes + ng * sl.bytes);
+                threads = std::max(threads, ng * T);
+            }
+            all = fit;
+        }
+        if (!all) continue;
+        lp.nz = NZ;
+        lp.smem_bytes = bytes;
+        block = threads;
+        grid = std::min(sms, std::max(1, zones));
+        ok = true;
+        return KN_OK;
     }
     return KN_OK;
 }
@@ -238,6 +321,17 @@ kn_status kn_check_gather_tables(const kn_network_desc* d, int32_t precision, in
     Tables T;
     s = build_tables_host(n.get(), precision, threads_per_zone, blob, T);
     if (s != KN_OK) return s;
+    if (precision == KN_PREC_MIXED && threads_per_zone >= n->N) {
+        // the tables of kn_slots.cu from the same summation order
+        const bool warp = threads_per_zone == 32;
+        const int cap = warp ? kCapWarp : (rate_cache_on(n.get(), kPrecMixed) ? kCapGroup : kCapEvery);
+        std::vector<unsigned char> sb;
+        SlotTables st;
+        bool fits;
+        for (int NZ = 1; NZ <= 2; ++NZ)
+            for (int W = warp ? 1 : (n->N + 31) / 32 + 1; W <= (warp ? 1 : kSlotThreads / 32); ++W)
+                if ((s = build_slots_host(n.get(), T, 32 * W, NZ, cap, sb, st, fits)) != KN_OK) return s;
+    }
     stats[0] = T.L;
     stats[1] = T.n_slices;
     stats[2] = T.warp_len;
@@ -413,6 +507,7 @@ static void set_guard_band(OptsDev& D, const kn_opts* o) {
     D.gb32 = (float)(o->safety * o->eps_c);
     D.grow32 = (float)o->grow_max;
     D.shrink32 = (float)o->shrink;
+    D.dt_min32 = (float)o->dt_min_frac;
     D.band_lo32 = (float)(1.0 - band);
     D.band_hi32 = (float)(1.0 + band);
     D.thr_lo32 = (float)(o->eps_r * (1.0 - band));
@@ -571,13 +666,23 @@ static kn_status prepare_launch(kn_network* const* nets, int n_nets, const kn_op
                         lp.plans[p].G * lp.plans[p].M, block);
     lp.smem_bytes = max_smem + (learn ? kMlpSmemBytes : 0);
     int bps = 0;
-    {
+    bool slots = false;
+    if (prec == kPrecMixed && !probe && !learn && !record && !o->replay_dt) {
+        s = plan_slots(nets, n_nets, tl, di.sms, budget, o->method == KN_METHOD_QSS, lp, grid, block, slots);
+        if (s != KN_OK) return s;
+        for (int p = 0; p < n_nets && slots; ++p) {
+            total_work -= work[p];
+            work[p] *= (double)tl[p].M / (lp.plans[p].ng * lp.nz);
+            total_work += work[p];
+        }
+    }
+    if (!slots) {
         cudaError_t e = integrator_occupancy(prec, block, lp.smem_bytes, &bps);
         if (e != cudaSuccess) return fail(KN_ERR_CUDA, "occupancy: %s", cudaGetErrorString(e));
+        if (bps < 1)
+            return fail(KN_ERR_INVALID_ARG, "tiling does not fit on an SM (block %d, smem %d)", block, lp.smem_bytes);
+        grid = di.sms * bps;
     }
-    if (bps < 1)
-        return fail(KN_ERR_INVALID_ARG, "tiling does not fit on an SM (block %d, smem %d)", block, lp.smem_bytes);
-    grid = di.sms * bps;
     int zones_total = 0;
     for (int p = 0; p < n_nets; ++p) zones_total += lp.plans[p].n_zones;
     if (probe) grid = std::min(grid, std::max(1, zones_total));
@@ -588,6 +693,7 @@ static kn_status prepare_launch(kn_network* const* nets, int n_nets, const kn_op
         cnt = std::max(0, std::min(cnt, grid - b));
         lp.plans[p].cta_begin = b;
         lp.plans[p].cta_end = b + cnt;
+        lp.plans[p].dealt = cnt * lp.plans[p].ng * lp.nz;
         b += cnt;
     }
     OptsDev& D = lp.o;
@@ -636,7 +742,7 @@ static kn_status prepare_launch(kn_network* const* nets, int n_nets, const kn_op
 static kn_status enqueue(kn_network* const* nets, int n_nets, const LaunchParams& lp, int prec, int grid,
                          int block, cudaStream_t st) {
     for (int p = 0; p < n_nets; ++p) KN_CUDA(cudaMemsetAsync(nets[p]->qhead.p, 0, sizeof(int), st));
-    KN_CUDA(launch_integrator(lp, prec, grid, block, st));
+    KN_CUDA(lp.nz ? launch_slots(lp, grid, block, st) : launch_integrator(lp, prec, grid, block, st));
     return KN_OK;
 }
 

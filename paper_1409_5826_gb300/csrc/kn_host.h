@@ -42,9 +42,27 @@ struct DevBuf {
     template <class T> T* as() const { return (T*)p; }
 };
 
+// The gather's summation order: the slices of 32 lanes, each lane's terms in order.
+struct GatherOrder {
+    struct Slice {
+        int len = 0;                  // terms per lane
+        std::vector<int> row;         // [32] the lane's row (F+_i: i, k_i: N + i; -1: no row)
+        std::vector<uint16_t> terms;  // [len][32] indices into V
+    };
+    std::vector<Slice> slices;
+};
+
+struct SlotBlob {
+    std::unique_ptr<DevBuf> blob;
+    SlotTables st{};
+    bool fits = false;
+};
+
 struct Tables {
     std::unique_ptr<DevBuf> blob;
     TableLayout tl{};
+    GatherOrder order;                               // mixed form
+    std::map<std::pair<int, int>, SlotBlob> slots;   // (threads, zones per group) -> device blob
     int L = 0, n_slices = 0, warp_len = 0;  // piece cap, slices, longest warp's terms per lane
 };
 }  // namespace kn
@@ -86,4 +104,11 @@ namespace kn {
 // checked on the host; `blob` is what goes to the device.
 kn_status network_host_setup(const kn_network_desc* d, std::unique_ptr<kn_network>& n, std::vector<double>& r0);
 kn_status build_tables_host(const kn_network* n, int prec, int Q, std::vector<unsigned char>& blob, Tables& T);
+// The slot tables (kn_slots.cu) for groups of T threads and NZ zones with the
+// capacities kSlotCaps[cap], from the summation order of `tb`; checked on the host
+// like the tables.  fits = false: the network does not fit the capacities or the
+// 16-bit offsets.
+kn_status build_slots_host(const kn_network* n, const Tables& tb, int T, int NZ, int cap, std::vector<unsigned char>& blob,
+                           SlotTables& st, bool& fits);
+SlotLayout slot_layout(const kn_network* n, const SlotTables& st, int T, int NZ, bool qss);
 }  // namespace kn

@@ -22,6 +22,7 @@
 #include <cstdint>
 #include <type_traits>
 
+#include "kn_device.cuh"
 #include "kn_internal.h"
 
 namespace kn {
@@ -41,18 +42,6 @@ struct GroupSync {
         }
     }
 };
-
-__device__ __forceinline__ long long global_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return (long long)t;
-}
-
-__device__ __forceinline__ float ex2_approx(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
 
 // exp(-x) for 0 <= x <= 2^-10 by its Taylor series (degree 5: the next term,
 // x^6/720, is below 2^-69 relative), or degree 2 for x <= 1e-6 (x^3/6 below
@@ -237,43 +226,6 @@ __device__ __forceinline__ void qss_predict(const PlanDev& P, const GroupPtrs& g
     for (int i = lane; i < N; i += G) Yp[i] = qss_update1(Yc[i], Fk[2 * i], Fk[2 * i + 1], h);
 }
 
-// FP32 versions for the mixed form.  In powers of r = 1/x above x = 1 the
-// c1 h f term is written (c1 / r) (f / k), since h r = 1/k: nothing then
-// overflows or underflows before the result does (x up to FLT_MAX).  The
-// denominators d and c2 lie in [1, 685], so the approximate division
-// __fdividef (2 ulp) is exact enough; f / k and 1/x use the correctly rounded
-// division and reciprocal.
-__device__ __forceinline__ void qss_weights32(float x, float& a, float& b) {
-    float n, d, dn;
-    if (x <= 1.f) {
-        n = fmaf(fmaf(x + 11.f, x, 60.f), x, 180.f);
-        d = fmaf(fmaf(x + 12.f, x, 60.f), x, 360.f);
-        dn = fmaf(x, x, 180.f);
-    } else {
-        const float r = __frcp_rn(x);
-        n = fmaf(fmaf(fmaf(180.f, r, 60.f), r, 11.f), r, 1.f);
-        d = fmaf(fmaf(fmaf(360.f, r, 60.f), r, 12.f), r, 1.f);
-        dn = r * fmaf(180.f * r, r, 1.f);
-    }
-    a = __fdividef(n, d);
-    b = __fdividef(dn, d);
-}
-
-__device__ __forceinline__ float qss_update1_32(float y, float f, float k, float h) {
-    const float x = __fmul_rn(k, h);
-    if (x <= 1.f) {
-        const float c0 = fmaf(fmaf(12.f, x, -120.f), x, 360.f);
-        const float c1 = fmaf(fmaf(x + 12.f, x, 60.f), x, 360.f);
-        const float c2 = fmaf(fmaf(fmaf(x + 12.f, x, 72.f), x, 240.f), x, 360.f);
-        return __fdividef(fmaf(c0, y, c1 * __fmul_rn(h, f)), c2);
-    }
-    const float r = __frcp_rn(x);
-    const float c0 = fmaf(fmaf(360.f, r, -120.f), r, 12.f) * __fmul_rn(r, r);
-    const float c1r = fmaf(fmaf(fmaf(360.f, r, 60.f), r, 12.f), r, 1.f);  // c1 / r
-    const float c2 = fmaf(fmaf(fmaf(fmaf(360.f, r, 240.f), r, 72.f), r, 12.f), r, 1.f);
-    return __fdividef(fmaf(c0, y, c1r * __fdiv_rn(f, k)), c2);
-}
-
 // Mixed form predictor: the FP32 copy of Yp (all the predicted state's flux
 // pass reads) into buffer nxt, from the high parts of the current pairs.
 __device__ __forceinline__ void qss_predict_mixed(const PlanDev& P, const GroupPtrs& g, int lane, int cur,
@@ -287,11 +239,6 @@ __device__ __forceinline__ void qss_predict_mixed(const PlanDev& P, const GroupP
         Yp[i] = qss_update1_32(Yh[i], fk.x, fk.y, h32);
     }
 }
-
-// Warps of a group that hold species (species i goes to lane i mod G): a warp
-// whose first lane is at or past N has none, skips the update and its
-// reductions, and is left out of the combine.
-__device__ __forceinline__ int species_warps(const PlanDev& P) { return (min(P.G, P.N) + 31) >> 5; }
 
 // (d) the update with step h from buffer cur into nxt, and each warp's share
 // of the error measures (no barrier inside).  FP64 form: every step in FP64,
@@ -354,15 +301,6 @@ __device__ __forceinline__ void update_reduce_fp64(const PlanDev& P, const OptsD
         g.red_n[w] = bn;
         g.red_d[w] = bd;
     }
-}
-
-// Knuth's TwoSum (TAOCP vol. 2, 4.2.2): s = fl(a + b) and the exact rounding
-// error e = (a + b) - s, for any a, b (no ordering condition).
-__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
-    s = __fadd_rn(a, b);
-    const float bv = __fsub_rn(s, a);
-    const float av = __fsub_rn(s, bv);
-    e = __fadd_rn(__fsub_rn(a, av), __fsub_rn(b, bv));
 }
 
 // Mixed form.  The abundances are float-float pairs y = yh + yl (|yl| at most

@@ -79,6 +79,46 @@ struct GroupLayout {
     int32_t off_state;  // GroupState
 };
 
+// The tables of the several-zones-per-group kernel (kn_slots.cu), one blob per
+// (group size of the summation order, threads, zones).  The gather's slices, row
+// pieces and term orders are those of TableLayout's list, dealt to the worker
+// warps; reactions are dealt to them by aligned blocks of 32.  A worker thread
+// loads its offsets once, into registers, so what it can hold is a compile-time
+// capacity.
+constexpr int kMaxSlots = 4;          // zones per group
+constexpr int kSlotThreads = 512;     // threads per CTA (128 registers each)
+constexpr int kSlotCtlBytes = 256;    // a group's scalars
+struct SlotCaps {
+    int f1, f2, fa;  // blocks of 1-body, 2-body and any reactions per thread
+    int ga, gb;      // words (two terms each) of a thread's two gather slices
+};
+enum { kCapWarp = 0, kCapGroup = 1, kCapEvery = 2, kCapMany = 3 };
+constexpr SlotCaps kSlotCaps[3] = {{0, 0, 2, 4, 4}, {3, 4, 2, 14, 8}, {4, 5, 2, 14, 10}};
+struct SlotTables {
+    int32_t bytes;      // the part staged in shared memory (multiple of 128): float[slots][Tw], c_j of each
+                        //   worker thread's blocks, then uint32[f1][Tw] at off_p0
+    int32_t off_p0;     // word offsets into V of the 1-body blocks' partials
+    int32_t off_words;  // uint32[..][Tw]: the words of Resident (kn_slots.cu), in its order
+    int32_t off_sj;     // uint16[slots][Tw]: the reaction of each worker thread's blocks (0xffff: none)
+    int32_t slots;      // f1 + f2 + fa
+    int32_t vrows;      // rows of 32 words of V
+    int32_t zero;       // V's constant 0, as a word offset (zone 0)
+};
+
+// A group's region (byte offsets).  Y and V hold word v of zone z at word
+// (v / 32) 32 NZ + 32 z + v % 32; the rates and the (F+, k) rows hold the zones'
+// values side by side.
+struct SlotLayout {
+    int32_t bytes;
+    int32_t off_V;    // fluxes, partials and the constant 0, placed by the tables
+    int32_t off_K;    // float[slots][Tw][NZ]: the zones' rates at (T0, rho0)
+    int32_t off_Y;    // the candidates' high parts, entry N the constant 1
+    int32_t off_Fk;   // float[N][2][NZ]: F+ of the zones, k of the zones
+    int32_t off_Fk2;  // the same of the QSS predicted state
+    int32_t off_red;  // float4[W][NZ]: a warp's conservation pair and maximum ratio; double[W] at write-back
+    int32_t off_ctl;  // SlotCtl
+};
+
 struct GroupState {
     double t, dt, t_end, h;
     double lnT0, lnR0, inv_tau, s;  // s = t / tau at the current step start
@@ -149,6 +189,12 @@ struct PlanDev {
     const int* order;            // work-queue order of zones (longest first)
     int* queue_head;             // work-queue counter (reset to 0 before each launch)
     int32_t cta_begin, cta_end;  // CTAs whose home is this plan
+    // kn_slots.cu
+    const unsigned char* slot_blob;
+    SlotTables st;
+    SlotLayout sl;
+    int32_t T, ng, cap;          // threads per group, groups per CTA, capacities
+    int32_t dealt;               // the first `dealt` zones of the queue go to the home CTAs' slots in turn
 };
 
 struct OptsDev {
@@ -182,6 +228,7 @@ struct OptsDev {
     float eps_r32, ymin_lo32, ymin_hi32, band_lo32, band_hi32, kappa32;
     float eps_c32, ga32, gb32, grow32;  // mixed form: eps_c and the growth factor's terms in FP32
     float shrink32;                     // mixed form: the reject factor in FP32
+    float dt_min32;                     // mixed form: dt_min_frac in FP32
     float thr_lo32, thr_hi32;           // mixed form: eps_r times the guard band's ends
     // trace of the learned proposal: features [cap][64], output [cap], dt record [cap][6]
     float* trace_feat;
@@ -200,6 +247,8 @@ struct OptsDev {
 struct LaunchParams {
     int32_t n_plans;
     int32_t smem_bytes;
+    int32_t nz;  // zones per group of kn_slots.cu; 0: the group kernel of kn_integrate.cu
+    int32_t pad;
     PlanDev plans[kMaxPlans];
     OptsDev o;
 };
@@ -207,6 +256,9 @@ struct LaunchParams {
 // Host-side launch of the integrator kernel (kn_integrate.cu).
 cudaError_t launch_integrator(const LaunchParams& lp, int precision, int grid, int block,
                               cudaStream_t stream);
+// Launch of the several-zones-per-group kernel (kn_slots.cu) and its shared-memory limit.
+cudaError_t launch_slots(const LaunchParams& lp, int grid, int block, cudaStream_t stream);
+cudaError_t slots_set_smem_limit(int bytes);
 // Occupancy query for a given precision, block size and shared memory.
 cudaError_t integrator_occupancy(int precision, int block, int smem, int* blocks_per_sm);
 // Enable the large dynamic shared memory carve-out for both kernel variants.

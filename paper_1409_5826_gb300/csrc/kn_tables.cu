@@ -2,6 +2,7 @@
 // validation, the sorted and bank-aware reaction order, the reactant table,
 // and the sliced gather list with its bank-aware term order and self-check.
 #include <algorithm>
+#include <array>
 #include <cmath>
 #include <cstring>
 #include <functional>
@@ -233,6 +234,7 @@ kn_status build_tables_host(const kn_network* n, int prec, int Q, std::vector<un
     const int vscale = byte_off ? real_bytes : 1;
     std::vector<uint32_t> shdr;
     int n_slices = 0;
+    T.order.slices.clear();
     for (int w = 0; w < W; ++w) {
         wsl[w] = (uint16_t)n_slices;
         for (int s : best.warp_slices[w]) {
@@ -250,6 +252,14 @@ kn_status build_tables_host(const kn_network* n, int prec, int Q, std::vector<un
             sidx.resize(base + 32 * (size_t)len, (uint16_t)(zero_idx * vscale));
             for (int l = 0; l < 32; ++l)
                 for (int k = 0; k < len; ++k) sidx[base + 32 * (size_t)k + l] = (uint16_t)(ordered[l][k] * vscale);
+            if (prec == kPrecMixed) {
+                GatherOrder::Slice os;
+                os.len = len;
+                for (int l = 0; l < 32; ++l) os.row.push_back(best.slices[s][l].row);
+                for (int k = 0; k < len; ++k)
+                    for (int l = 0; l < 32; ++l) os.terms.push_back(ordered[l][k]);
+                T.order.slices.push_back(std::move(os));
+            }
             ++n_slices;
         }
     }
@@ -352,6 +362,373 @@ kn_status build_tables_host(const kn_network* n, int prec, int Q, std::vector<un
     return KN_OK;
 }
 
+
+SlotLayout slot_layout(const kn_network* n, const SlotTables& st, int T, int NZ, bool qss) {
+    const int W = T / 32, Tw = T > 32 ? T - 32 : 32;
+    SlotLayout l{};
+    int off = 0;
+    l.off_V = off;
+    off += 128 * NZ * st.vrows;
+    l.off_Y = off;
+    off += 128 * NZ * ((n->N + 32) / 32);
+    l.off_K = off;
+    off += 4 * NZ * Tw * st.slots;
+    l.off_Fk = off;
+    off = pad16(off + 8 * NZ * n->N);
+    l.off_Fk2 = off;
+    if (qss) off = pad16(off + 8 * NZ * n->N);
+    l.off_red = off;
+    off += 16 * W * NZ;
+    l.off_ctl = off;
+    off += kSlotCtlBytes;
+    l.bytes = (off + 127) & ~127;  // the next group's interleaved arrays start at bank 0
+    return l;
+}
+
+namespace {
+// Banks for V's values.  A value is stored by one warp instruction (a block's 32
+// lanes, one plane) and loaded by one to three (a gather step); each takes one
+// wavefront when its distinct words lie in distinct banks.  Minimum-conflicts
+// search: sweeps over the values, each moving to the bank with the fewest values
+// of its instructions (then the emptiest one), with a bound on a bank's values.
+static std::vector<int> place_banks(int nv, const std::vector<std::vector<int>>& groups, int rows) {
+    std::vector<std::vector<int>> of(nv);
+    for (int g = 0; g < (int)groups.size(); ++g)
+        for (int v : groups[g]) of[v].push_back(g);
+    std::vector<int> bank(nv, -1), fill(32, 0);
+    std::vector<std::array<uint8_t, 32>> cnt(groups.size());
+    for (auto& c : cnt) c.fill(0);
+    uint32_t rng = 12345;
+    auto best_bank = [&](int v) {
+        int best = -1, cost = 1 << 30;
+        rng = rng * 1664525u + 1013904223u;
+        const int start = (int)(rng >> 27);
+        for (int i = 0; i < 32; ++i) {
+            const int b = (start + i) & 31;
+            if (fill[b] >= rows) continue;
+            int c = 0;
+            for (int g : of[v]) c += cnt[g][b];
+            c = c * 4096 + fill[b];
+            if (c < cost) {
+                cost = c;
+                best = b;
+            }
+        }
+        return best;
+    };
+    auto put = [&](int v, int b, int d) {
+        fill[b] += d;
+        for (int g : of[v]) cnt[g][b] = (uint8_t)(cnt[g][b] + d);
+    };
+    for (int v = 0; v < nv; ++v) {
+        bank[v] = best_bank(v);
+        put(v, bank[v], 1);
+    }
+    for (int sweep = 0; sweep < 40; ++sweep) {
+        int moved = 0;
+        for (int v = 0; v < nv; ++v) {
+            int own = 0;
+            for (int g : of[v]) own += cnt[g][bank[v]] - 1;
+            if (!own) continue;
+            put(v, bank[v], -1);
+            const int b = best_bank(v);
+            moved += b != bank[v];
+            bank[v] = b;
+            put(v, b, 1);
+        }
+        if (!moved) break;
+    }
+    return bank;
+}
+}  // namespace
+
+kn_status build_slots_host(const kn_network* n, const Tables& tb, int T, int NZ, int cap, std::vector<unsigned char>& blob,
+                           SlotTables& st, bool& fits) {
+    fits = false;
+    st = SlotTables{};
+    const SlotCaps C = kSlotCaps[cap];
+    const int N = n->N, R = n->R, W = T / 32, Ww = W > 1 ? W - 1 : 1, Tw = 32 * Ww, blocks = (R + 31) / 32,
+              zero_idx = R + n->S_r;
+    auto word = [NZ](int v) { return v / 32 * 32 * NZ + v % 32; };
+    if (word(N) > 0xffff || 8 * NZ * N > 0xffff) return KN_OK;
+    // ---- gather slices to workers: at most two each, the longest first to the
+    // least loaded (costs in terms: set-up 6, a reduction round 2) ----
+    const int ns = (int)tb.order.slices.size();
+    std::vector<int> rounds(ns, 0), cost(ns), ord(ns);
+    for (int s = 0; s < ns; ++s) {
+        const auto& sl = tb.order.slices[s];
+        int most = 1;
+        for (int l = 0; l < 32;) {
+            int e = l + 1;
+            while (e < 32 && sl.row[l] >= 0 && sl.row[e] == sl.row[l]) ++e;
+            most = std::max(most, e - l);
+            l = e;
+        }
+        while ((1 << rounds[s]) < most) ++rounds[s];
+        cost[s] = 6 + sl.len + 2 * rounds[s];
+        ord[s] = s;
+    }
+    std::stable_sort(ord.begin(), ord.end(), [&](int x, int y) { return cost[x] > cost[y]; });
+    if (ns > 2 * Ww) return KN_OK;
+    std::vector<std::vector<int>> mine(Ww);
+    std::vector<int> load(Ww, 0);
+    for (int s : ord) {
+        int w = -1;
+        for (int i = 0; i < Ww; ++i)
+            if (mine[i].size() < 2 && (w < 0 || load[i] < load[w])) w = i;
+        // the first slice of a warp is its longest; the second has the smaller capacity
+        if ((tb.order.slices[s].len + 3) / 4 * 2 > (mine[w].empty() ? C.ga : C.gb)) return KN_OK;
+        mine[w].push_back(s);
+        load[w] += cost[s];
+    }
+    // ---- blocks of reactions to workers: whole 1- and 2-body blocks to their own
+    // slots, the others (and what overflows) to the slots for any block ----
+    struct Bl {
+        int b, cls, cost;
+    };
+    std::vector<Bl> bl;
+    for (int b = 0; b < blocks; ++b) {
+        const int j0 = 32 * b, j1 = j0 + 31;
+        int cls = 3;
+        if (j1 < n->R1) cls = 1;
+        else if (j0 >= n->R1 && j1 < n->R12) cls = 2;
+        bl.push_back({b, cls, cls == 1 ? 8 : (cls == 2 ? 19 : 30)});
+    }
+    std::stable_sort(bl.begin(), bl.end(), [](const Bl& x, const Bl& y) { return x.cost > y.cost; });
+    std::vector<std::vector<int>> k1(Ww), k2(Ww), ka(Ww);
+    std::vector<int> fl(Ww, 0);
+    for (const Bl& x : bl) {
+        int w = -1, to = 0;
+        for (int pass = 0; pass < 2 && w < 0; ++pass)  // its own sort of slot, then any
+            for (int i = 0; i < Ww; ++i) {
+                const int t = pass == 0 ? x.cls : 3;
+                const bool room = t == 1 ? (int)k1[i].size() < C.f1 : (t == 2 ? (int)k2[i].size() < C.f2 : (int)ka[i].size() < C.fa);
+                if (room && (w < 0 || fl[i] < fl[w])) {
+                    w = i;
+                    to = t;
+                }
+            }
+        if (w < 0) return KN_OK;
+        (to == 1 ? k1 : (to == 2 ? k2 : ka))[w].push_back(x.b);
+        fl[w] += to == 3 ? 30 : x.cost;
+    }
+    // ---- V: banks for the values, from the instructions that store and load them ----
+    const int plane[3] = {R, 2 * R - n->R1, 3 * R - n->R1 - n->R12};
+    std::vector<std::vector<int>> groups;
+    for (int b = 0; b < blocks; ++b)
+        for (int q = 0; q < 4; ++q) {
+            std::vector<int> g;
+            for (int j = 32 * b; j < std::min(R, 32 * b + 32); ++j) {
+                const int nr = n->nr[n->perm[j]];
+                if (q == 0) g.push_back(j);
+                else if (q <= nr) g.push_back(plane[q - 1] + j);
+            }
+            if (!g.empty()) groups.push_back(std::move(g));
+        }
+    for (const auto& sl : tb.order.slices)
+        for (int k = 0; k < sl.len; ++k) {
+            std::vector<int> g;
+            for (int l = 0; l < 32; ++l) {
+                const int v = sl.terms[32 * (size_t)k + l];
+                if (v != zero_idx && std::find(g.begin(), g.end(), v) == g.end()) g.push_back(v);
+            }
+            groups.push_back(std::move(g));
+        }
+    st.vrows = (zero_idx + 1 + 31) / 32 + 1;
+    const std::vector<int> bank = place_banks(zero_idx, groups, st.vrows - 1);
+    std::vector<int> at(zero_idx + 1), next(32, 0);
+    for (int v = 0; v < zero_idx; ++v) at[v] = 32 * NZ * next[bank[v]]++ + bank[v];
+    at[zero_idx] = 32 * NZ * (st.vrows - 1);
+    st.zero = at[zero_idx];
+    if (32 * NZ * st.vrows > 0x10000) return KN_OK;
+    // ---- the words ----
+    st.slots = C.f1 + C.f2 + C.fa;
+    const int nwords = C.f1 + 3 * C.f2 + 4 * C.fa + C.ga + C.gb + 3;
+    std::vector<uint32_t> wd((size_t)nwords * Tw, 0), p0((size_t)C.f1 * Tw, 0);
+    std::vector<uint16_t> sj((size_t)st.slots * Tw, 0xffff);
+    std::vector<float> ce((size_t)st.slots * Tw, 0.f);
+    for (int w = 0; w < Ww; ++w)
+        for (int l = 0; l < 32; ++l) {
+            const int t = 32 * w + l;
+            auto set = [&](int i, uint32_t lo, uint32_t hi) { wd[(size_t)i * Tw + t] = lo | hi << 16; };
+            auto fill = [&](int slot, int jn, uint32_t (&a)[8]) {  // a, b, c; V, P0, P1, P2; reactants
+                for (int q = 0; q < 8; ++q) a[q] = q < 3 ? (uint32_t)word(N) : 0;
+                if (jn >= R) return;
+                const int j = n->perm[jn];
+                for (int q = 0; q < n->nr[j]; ++q) a[q] = (uint32_t)word(n->reac[j * 3 + q]);
+                a[3] = (uint32_t)at[jn];
+                for (int q = 0; q < n->nr[j]; ++q) a[4 + q] = (uint32_t)at[plane[q] + jn];
+                a[7] = (uint32_t)n->nr[j];
+                sj[(size_t)slot * Tw + t] = (uint16_t)jn;
+                ce[(size_t)slot * Tw + t] = (float)(n->tn[j] + 3.0 * (n->nr[j] - 1));
+            };
+            uint32_t a[8];
+            int i = 0;
+            for (int k = 0; k < C.f1; ++k, ++i)
+                if (k < (int)k1[w].size()) {
+                    fill(k, 32 * k1[w][k] + l, a);
+                    set(i, a[0], a[3]);
+                    p0[(size_t)k * Tw + t] = a[4];
+                }
+            for (int k = 0; k < C.f2; ++k, i += 3)
+                if (k < (int)k2[w].size()) {
+                    fill(C.f1 + k, 32 * k2[w][k] + l, a);
+                    set(i, a[0], a[1]);
+                    set(i + 1, a[3], a[4]);
+                    set(i + 2, a[5], 0);
+                }
+            for (int k = 0; k < C.fa; ++k, i += 4)
+                if (k < (int)ka[w].size()) {
+                    fill(C.f1 + C.f2 + k, 32 * ka[w][k] + l, a);
+                    set(i, a[0], a[1]);
+                    set(i + 1, a[2], a[3]);
+                    set(i + 2, a[4], a[5]);
+                    set(i + 3, a[6], a[7]);
+                }
+            uint32_t cnt = (uint32_t)k1[w].size() | (uint32_t)k2[w].size() << 4 | (uint32_t)ka[w].size() << 8;
+            uint32_t dst[2] = {0, 0};
+            for (int h = 0; h < 2; ++h) {
+                const int room = h ? C.gb : C.ga;
+                const bool has = h < (int)mine[w].size();
+                if (has) {
+                    const auto& sl = tb.order.slices[mine[w][h]];
+                    // lengths rounded up to four by the constant 0 (adding +0 changes no
+                    // sum of non-negative terms)
+                    for (int k = 0; k < room; ++k) {
+                        auto term = [&](int q) { return (uint32_t)at[q < sl.len ? sl.terms[32 * (size_t)q + l] : zero_idx]; };
+                        set(i + k, term(2 * k), term(2 * k + 1));
+                    }
+                    const int rd = rounds[mine[w][h]], r = sl.row[l];
+                    if (r >= 0) {
+                        uint32_t d = (uint32_t)(8 * NZ * (r % N) + (r >= N ? 4 * NZ : 0));
+                        if (l == 0 || sl.row[l - 1] != r) d |= 1u << 16;
+                        for (int q = 0; q < rd; ++q)
+                            if (l + (1 << q) < 32 && sl.row[l + (1 << q)] == r) d |= 1u << (17 + q);
+                        dst[h] = d;
+                    }
+                    cnt |= (uint32_t)((sl.len + 3) / 4 * 2) << (h ? 18 : 12) | (uint32_t)rd << (h ? 28 : 24);
+                }
+                i += room;
+            }
+            wd[(size_t)i * Tw + t] = dst[0];
+            wd[(size_t)(i + 1) * Tw + t] = dst[1];
+            wd[(size_t)(i + 2) * Tw + t] = cnt;
+        }
+    // ---- host check, through the words: every reaction in one thread's block with
+    // its reactants and its places in V, and the gather with V[v] = v + 1 giving
+    // every row once ----
+    {
+        std::vector<double> V((size_t)32 * NZ * st.vrows, -1.0);
+        std::vector<char> seen(R, 0);
+        const int gaw = C.f1 + 3 * C.f2 + 4 * C.fa;
+        for (int t = 0; t < Tw; ++t) {
+            const uint32_t cnt = wd[(size_t)(nwords - 1) * Tw + t];
+            auto wrd = [&](int i) { return wd[(size_t)i * Tw + t]; };
+            for (int sl = 0; sl < st.slots; ++sl) {
+                const int jn = sj[(size_t)sl * Tw + t];
+                if (jn == 0xffff) continue;
+                if (jn >= R || seen[jn]++) return fail(KN_ERR_INTERNAL, "slot tables: reaction %d dealt twice", jn);
+                const int j = n->perm[jn], nr = n->nr[j];
+                uint32_t y[3] = {(uint32_t)word(N), (uint32_t)word(N), (uint32_t)word(N)}, p[4] = {0, 0, 0, 0};
+                int used;
+                if (sl < C.f1) {
+                    used = 1;
+                    y[0] = wrd(sl) & 0xffff;
+                    p[0] = wrd(sl) >> 16;
+                    p[1] = p0[(size_t)sl * Tw + t];
+                    if (sl >= (int)(cnt & 15)) return fail(KN_ERR_INTERNAL, "slot tables: block count");
+                } else if (sl < C.f1 + C.f2) {
+                    used = 2;
+                    const int i = C.f1 + 3 * (sl - C.f1);
+                    y[0] = wrd(i) & 0xffff;
+                    y[1] = wrd(i) >> 16;
+                    p[0] = wrd(i + 1) & 0xffff;
+                    p[1] = wrd(i + 1) >> 16;
+                    p[2] = wrd(i + 2);
+                    if (sl - C.f1 >= (int)(cnt >> 4 & 15)) return fail(KN_ERR_INTERNAL, "slot tables: block count");
+                } else {
+                    const int i = C.f1 + 3 * C.f2 + 4 * (sl - C.f1 - C.f2);
+                    y[0] = wrd(i) & 0xffff;
+                    y[1] = wrd(i) >> 16;
+                    y[2] = wrd(i + 1) & 0xffff;
+                    p[0] = wrd(i + 1) >> 16;
+                    p[1] = wrd(i + 2) & 0xffff;
+                    p[2] = wrd(i + 2) >> 16;
+                    p[3] = wrd(i + 3) & 0xffff;
+                    used = (int)(wrd(i + 3) >> 16);
+                    if (sl - C.f1 - C.f2 >= (int)(cnt >> 8 & 15)) return fail(KN_ERR_INTERNAL, "slot tables: block count");
+                }
+                if (used != nr) return fail(KN_ERR_INTERNAL, "slot tables: reactants of reaction %d", jn);
+                for (int q = 0; q < 3; ++q)
+                    if ((int)y[q] != word(q < nr ? n->reac[j * 3 + q] : N)) return fail(KN_ERR_INTERNAL, "slot tables: reactant");
+                for (int q = 0; q <= nr; ++q) {
+                    if (p[q] >= V.size() || p[q] % (32 * NZ) >= 32 || V[p[q]] >= 0.0)
+                        return fail(KN_ERR_INTERNAL, "slot tables: a value's place");
+                    V[p[q]] = (q == 0 ? jn : plane[q - 1] + jn) + 1.0;
+                }
+            }
+        }
+        for (int j = 0; j < R; ++j)
+            if (!seen[j]) return fail(KN_ERR_INTERNAL, "slot tables: reaction %d not dealt", j);
+        if (V[st.zero] >= 0.0) return fail(KN_ERR_INTERNAL, "slot tables: the constant 0's place");
+        V[st.zero] = 0.0;
+        std::vector<double> got(2 * (size_t)N, -1.0), want(2 * (size_t)N, 0.0);
+        for (const auto& sl : tb.order.slices)
+            for (int k = 0; k < sl.len; ++k)
+                for (int l = 0; l < 32; ++l)
+                    if (sl.row[l] >= 0 && sl.terms[32 * (size_t)k + l] != zero_idx)
+                        want[sl.row[l]] += sl.terms[32 * (size_t)k + l] + 1.0;
+        for (int w = 0; w < Ww; ++w)
+            for (int h = 0; h < 2; ++h) {
+                double acc[32];
+                uint32_t d[32];
+                int rd = 0;
+                for (int l = 0; l < 32; ++l) {
+                    const int t = 32 * w + l;
+                    const uint32_t cnt = wd[(size_t)(nwords - 1) * Tw + t];
+                    const int words = (int)(cnt >> (h ? 18 : 12) & 63);
+                    rd = (int)(h ? cnt >> 28 : cnt >> 24 & 7);
+                    d[l] = words ? wd[(size_t)(nwords - 3 + h) * Tw + t] : 0;
+                    acc[l] = 0.0;
+                    for (int k = 0; k < words; ++k) {
+                        const uint32_t x = wd[(size_t)(gaw + (h ? C.ga : 0) + k) * Tw + t];
+                        for (uint32_t v : {x & 0xffffu, x >> 16}) {
+                            if (v >= V.size() || V[v] < 0.0) return fail(KN_ERR_INTERNAL, "slot tables: term out of range");
+                            acc[l] += V[v];
+                        }
+                    }
+                }
+                for (int r = 0; r < rd; ++r)
+                    for (int l = 0; l < 32; ++l)  // ascending: the lane up still holds the last round's sum
+                        if (d[l] >> (17 + r) & 1) acc[l] += acc[l + (1 << r)];
+                for (int l = 0; l < 32; ++l) {
+                    if (!(d[l] >> 16 & 1)) continue;
+                    const int o = (int)(d[l] & 0xffffu), i = o / (8 * NZ), q = o % (8 * NZ);
+                    if (i >= N || (q != 0 && q != 4 * NZ)) return fail(KN_ERR_INTERNAL, "slot tables: bad destination");
+                    double& x = got[(q ? N : 0) + i];
+                    if (x >= 0.0) return fail(KN_ERR_INTERNAL, "slot tables: row stored twice");
+                    x = acc[l];
+                }
+            }
+        for (int r = 0; r < 2 * N; ++r)
+            if (got[r] != want[r]) return fail(KN_ERR_INTERNAL, "slot tables: row %d sums to %g, not %g", r, got[r], want[r]);
+    }
+    int off = 4 * (int)ce.size();
+    st.off_p0 = off;
+    off += 4 * (int)p0.size();
+    st.bytes = off = (off + 127) & ~127;
+    st.off_words = off;
+    off += 4 * (int)wd.size();
+    st.off_sj = off;
+    off += 2 * (int)sj.size();
+    blob.assign(off, 0);
+    memcpy(blob.data(), ce.data(), 4 * ce.size());
+    memcpy(blob.data() + st.off_p0, p0.data(), 4 * p0.size());
+    memcpy(blob.data() + st.off_words, wd.data(), 4 * wd.size());
+    memcpy(blob.data() + st.off_sj, sj.data(), 2 * sj.size());
+    fits = true;
+    return KN_OK;
+}
 
 // Validation, the sorted reaction order and the host-side network data; no
 // device work.
