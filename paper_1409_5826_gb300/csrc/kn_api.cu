@@ -179,7 +179,7 @@ static kn_status plan_tiling(kn_network* n, int prec, int P, int budget, int G_f
 // The slot tables of one network for (G, T, NZ, cap), built on first use.
 static kn_status get_slots(kn_network* n, int G, int T, int NZ, int cap, SlotBlob** out) {
     Tables& tb = n->tables.at({kPrecMixed, G});
-    auto it = tb.slots.find({T, NZ});
+    auto it = tb.slots.find({T, 8 * NZ + cap});
     if (it == tb.slots.end()) {
         std::vector<unsigned char> blob;
         SlotBlob sb;
@@ -190,7 +190,7 @@ static kn_status get_slots(kn_network* n, int G, int T, int NZ, int cap, SlotBlo
             KN_CUDA(sb.blob->ensure(blob.size()));
             KN_CUDA(cudaMemcpy(sb.blob->p, blob.data(), blob.size(), cudaMemcpyHostToDevice));
         }
-        it = tb.slots.emplace(std::make_pair(T, NZ), std::move(sb)).first;
+        it = tb.slots.emplace(std::make_pair(T, 8 * NZ + cap), std::move(sb)).first;
     }
     *out = &it->second;
     return KN_OK;
@@ -219,22 +219,21 @@ static kn_status plan_slots(kn_network* const* nets, int n_nets, const Tiling* t
             PlanDev& P = lp.plans[p];
             const bool warp = tl[p].G == 32;
             if (warp && !rate_cache_on(n, kPrecMixed)) return KN_OK;
-            const int cap = warp ? kCapWarp : (rate_cache_on(n, kPrecMixed) ? kCapGroup : kCapEvery);
-            // the most groups that the zones can use, each of at least the species'
-            // warps and the one that decides, then all threads to those groups
+            // the most groups that the zones can use (three at most: fewer groups of
+            // more threads step faster, 100 species 32 against 38 ms at two of 256 and
+            // three of 160), each of at least the species' warps and the one that
+            // decides, then all threads to those groups
             const int lo = warp ? 32 : (n->N + 31) / 32 * 32 + 32;
-            int ng = std::min(warp ? kSlotThreads / 32 : kMaxGroups, kSlotThreads / lo);
-            ng = std::max(1, std::min(ng, (zps + NZ - 1) / NZ));
+            const int most = std::max(1, std::min({warp ? kSlotThreads / 32 : 3, kSlotThreads / lo, (zps + NZ - 1) / NZ}));
             bool fit = false;
-            for (; ng >= 1 && !fit; --ng) {
+            auto try_plan = [&](int cap, int ng) -> kn_status {
                 const int T = warp ? 32 : kSlotThreads / ng / 32 * 32;
-                if (T < lo) continue;
+                if (T < lo) return KN_OK;
                 SlotBlob* sb;
                 kn_status s = get_slots(n, tl[p].G, T, NZ, cap, &sb);
-                if (s != KN_OK) return s;
-                if (!sb->fits) continue;
+                if (s != KN_OK || !sb->fits) return s;
                 const SlotLayout sl = slot_layout(n, sb->st, T, NZ, qss);
-                if (sb->st.bytes + ng * sl.bytes > budget) continue;
+                if (sb->st.bytes + ng * sl.bytes > budget) return KN_OK;
                 P.slot_blob = (const unsigned char*)sb->blob->p;
                 P.st = sb->st;
                 P.sl = sl;
@@ -244,7 +243,13 @@ static kn_status plan_slots(kn_network* const* nets, int n_nets, const Tiling* t
                 fit = true;
                 bytes = std::max(bytes, P.st.bytes + ng * sl.bytes);
                 threads = std::max(threads, ng * T);
-            }
+                return KN_OK;
+            };
+            for (int cap = warp ? kCapWarp : kCapGroup; cap <= (warp ? kCapWarp : kCapWide) && !fit; ++cap)
+                for (int ng = most; ng >= 1 && !fit; --ng) {
+                    const kn_status s = try_plan(cap, ng);
+                    if (s != KN_OK) return s;
+                }
             all = fit;
         }
         if (!all) continue;
@@ -324,13 +329,13 @@ kn_status kn_check_gather_tables(const kn_network_desc* d, int32_t precision, in
     if (precision == KN_PREC_MIXED && threads_per_zone >= n->N) {
         // the tables of kn_slots.cu from the same summation order
         const bool warp = threads_per_zone == 32;
-        const int cap = warp ? kCapWarp : (rate_cache_on(n.get(), kPrecMixed) ? kCapGroup : kCapEvery);
         std::vector<unsigned char> sb;
         SlotTables st;
         bool fits;
         for (int NZ = 1; NZ <= 2; ++NZ)
             for (int W = warp ? 1 : (n->N + 31) / 32 + 1; W <= (warp ? 1 : kSlotThreads / 32); ++W)
-                if ((s = build_slots_host(n.get(), T, 32 * W, NZ, cap, sb, st, fits)) != KN_OK) return s;
+                for (int cap = warp ? kCapWarp : kCapGroup; cap <= (warp ? kCapWarp : kCapWide); ++cap)
+                    if ((s = build_slots_host(n.get(), T, 32 * W, NZ, cap, sb, st, fits)) != KN_OK) return s;
     }
     stats[0] = T.L;
     stats[1] = T.n_slices;
@@ -450,6 +455,10 @@ namespace {
 static float rate_cache_tol(double cmax) {
     return cmax > 0.0 ? (float)(1.4901161193847656e-08 / (cmax * 0.6931471805599453)) : 3.0e38f;
 }
+
+// ex2.approx(x) is 1 for every FP32 |x| <= 2^-26 (all of them tried on an sm_103
+// device); fl(c u) stays below that while |u| <= 2^-27 / c_max.
+static float one_tol(double cmax) { return cmax > 0.0 ? (float)(7.450580596923828e-09 / cmax) : 3.0e38f; }
 
 // Which autotuned tiling a call uses: the plain form's, the learned form's or
 // the QSS form's (they differ in shared memory per group and in work per step).
@@ -624,6 +633,7 @@ static kn_status prepare_launch(kn_network* const* nets, int n_nets, const kn_op
         P.R12 = n->R12;
         P.cmax = n->cmax;
         P.u_tol = rate_cache_tol(n->cmax);
+        P.u_one = one_tol(n->cmax);
         P.rate_cache = rate_cache_on(n, prec) ? 1 : 0;
         P.N = n->N;
         P.R = n->R;

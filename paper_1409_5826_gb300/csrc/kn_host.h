@@ -62,7 +62,7 @@ struct Tables {
     std::unique_ptr<DevBuf> blob;
     TableLayout tl{};
     GatherOrder order;                               // mixed form
-    std::map<std::pair<int, int>, SlotBlob> slots;   // (threads, zones per group) -> device blob
+    std::map<std::pair<int, int>, SlotBlob> slots;   // (threads, 8 zones per group + capacities) -> device blob
     int L = 0, n_slices = 0, warp_len = 0;  // piece cap, slices, longest warp's terms per lane
 };
 }  // namespace kn

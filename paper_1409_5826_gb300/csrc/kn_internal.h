@@ -92,8 +92,8 @@ struct SlotCaps {
     int f1, f2, fa;  // blocks of 1-body, 2-body and any reactions per thread
     int ga, gb;      // words (two terms each) of a thread's two gather slices
 };
-enum { kCapWarp = 0, kCapGroup = 1, kCapEvery = 2, kCapMany = 3 };
-constexpr SlotCaps kSlotCaps[3] = {{0, 0, 2, 4, 4}, {3, 4, 2, 14, 8}, {4, 5, 2, 14, 10}};
+enum { kCapWarp = 0, kCapGroup = 1, kCapWide = 2, kCapMany = 3 };
+constexpr SlotCaps kSlotCaps[3] = {{0, 0, 2, 4, 2}, {3, 4, 1, 14, 6}, {4, 5, 2, 14, 10}};
 struct SlotTables {
     int32_t bytes;      // the part staged in shared memory (multiple of 128): float[slots][Tw], c_j of each
                         //   worker thread's blocks, then uint32[f1][Tw] at off_p0
@@ -163,6 +163,7 @@ struct PlanDev {
     double cmax;                 // max_j c_j
     float u_tol;                 // FP32-flux forms: cached rates are reused while |u - u_ref| <= u_tol,
                                  //   i.e. while no rate would move by a quarter ulp: 2^-26 / (cmax ln 2)
+    float u_one;                 // kn_slots.cu without the rate cache: 2^(-c u) rounds to 1 while |u| <= u_one
     int32_t rate_cache;          // 1: the groups keep the cache Kc (FP32-flux forms, small enough R)
     int32_t zero_idx;            // V index of the constant zero (= R + S_r)
     int32_t smem_tables;         // 1: stage blob into shared memory

@@ -171,7 +171,8 @@ template <int NZ> __device__ __forceinline__ int at(int v) { return (v >> 5) * (
 // control warp (a single-warp group keeps them in registers)
 // ---------------------------------------------------------------------------
 struct Scal {
-    double t, te, ta;        // time, end, the time an accept reaches
+    double t, te, ts, ta;    // time, end, t + h, the time an accept reaches
+    double rem_d;            // te - ta
     long long steps, rejects;
     float h, dt;             // the attempt's step, the controller's next one
     float rem, rem_acc;      // te - t, te - ta
@@ -263,61 +264,62 @@ template <int NZ, class CAP> struct Resident {
     }
 };
 
-// a thread's shared addresses
+// shared addresses of the group's V, Y and scalars
 struct WorkAddr {
-    uint32_t V, Y, K, c, p0, ctl;  // K, c, p0: of this thread's block 0; block i: i strides further
-    int Kst, cst;
+    uint32_t V, Y, ctl;
 };
-template <int NZ> __device__ __forceinline__ WorkAddr work_addr(const PlanDev& P, const SlotBase& g, int wt, int Tw) {
-    return WorkAddr{g.gb + P.sl.off_V, g.gb + P.sl.off_Y, g.gb + P.sl.off_K + 4 * NZ * wt, g.tb + 4 * wt,
-                    g.tb + P.st.off_p0 + 4 * wt, g.gb + P.sl.off_ctl, 4 * NZ * Tw, 4 * Tw};
+__device__ __forceinline__ WorkAddr work_addr(const PlanDev& P, const SlotBase& g) {
+    return WorkAddr{g.gb + P.sl.off_V, g.gb + P.sl.off_Y, g.gb + P.sl.off_ctl};
 }
 
-// the rates K 2^(-c u) of block i's reaction in the zones of `mask`
-template <int NZ>
-__device__ __forceinline__ void rates_of(const WorkAddr& f, int i, uint32_t mask, typename Pack<NZ>::T (&k)[Pack<NZ>::n]) {
-    const float c = lds(f.c + i * f.cst);
-#pragma unroll
-    for (int z = 0; z < NZ; ++z)
-        if (mask >> z & 1)
-            zset<NZ>(k, z, __fmul_rn(lds(f.K + i * f.Kst + 4 * z),
-                                     ex2_approx(-__fmul_rn(c, lds(f.ctl + 32 + 4 * z)))));  // SlotCtl::u
-}
-
-// the cached rates of the zones of `mask`, at the u set for them; a 1-body
-// reaction's partial is its rate, so it is stored here and nowhere else
+// The cached rates K 2^(-c u) of the zones of `mask`, at the u set for them.  A
+// 1-body reaction's partial is its rate, so it is stored here and nowhere else.
+// wt: the worker thread, Tw of them.
 template <int NZ, class CAP>
-__device__ __forceinline__ void refresh_rates(Resident<NZ, CAP>& r, const WorkAddr& f, uint32_t mask) {
-    const int n1 = r.cnt & 15, n2 = r.cnt >> 4 & 15, na = r.cnt >> 8 & 15;
+__device__ __forceinline__ void refresh_rates(const PlanDev& P, const SlotBase& g, int wt, int Tw, Resident<NZ, CAP>& r,
+                                              const WorkAddr& f, uint32_t mask) {
+    using PK = typename Pack<NZ>::T;
+    constexpr int n = Pack<NZ>::n;
+    // opaque: the blocks' addresses are formed here, not kept through the step loop
+    asm volatile("" : "+r"(wt), "+r"(Tw));
+    uint32_t c = g.tb + 4 * wt, K = g.gb + P.sl.off_K + 4 * NZ * wt, p0 = g.tb + P.st.off_p0 + 4 * wt;
+    const int n1 = r.cnt & 15, n2 = r.cnt >> 4 & 15, na = r.cnt >> 8 & 15, cs = 4 * Tw, Ks = 4 * NZ * Tw;
+    float u[NZ];
 #pragma unroll
-    for (int i = 0; i < CAP::F1; ++i)
+    for (int z = 0; z < NZ; ++z) u[z] = lds(f.ctl + 32 + 4 * z);  // SlotCtl::u
+    auto rates = [&](PK (&k)[n]) {
+        const float cj = lds(c);
+        PK k0[n];
+#pragma unroll
+        for (int q = 0; q < n; ++q) ldp(K + (int)sizeof(PK) * q, k0[q]);
+#pragma unroll
+        for (int z = 0; z < NZ; ++z)
+            if (mask >> z & 1) zset<NZ>(k, z, __fmul_rn(zget<NZ>(k0, z), ex2_approx(-__fmul_rn(cj, u[z]))));
+    };
+#pragma unroll
+    for (int i = 0; i < CAP::F1; ++i, c += cs, K += Ks, p0 += cs)
         if (i < n1) {
-            rates_of<NZ>(f, i, mask, r.k1[i]);
-            st_zones<NZ>(f.V + 4 * ldu(f.p0 + i * f.cst), r.k1[i]);
+            rates(r.k1[i]);
+            st_zones<NZ>(f.V + 4 * ldu(p0), r.k1[i]);
         }
 #pragma unroll
-    for (int i = 0; i < CAP::F2; ++i)
-        if (i < n2) rates_of<NZ>(f, CAP::F1 + i, mask, r.k2[i]);
+    for (int i = 0; i < CAP::F2; ++i, c += cs, K += Ks)
+        if (i < n2) rates(r.k2[i]);
 #pragma unroll
-    for (int i = 0; i < CAP::FA; ++i)
-        if (i < na) rates_of<NZ>(f, CAP::F1 + CAP::F2 + i, mask, r.ka[i]);
+    for (int i = 0; i < CAP::FA; ++i, c += cs, K += Ks)
+        if (i < na) rates(r.ka[i]);
 }
 
 // (a) rates, fluxes and reactant-slot partials (Eq. 1) of the states at Y
-template <int NZ, bool EVERY, class CAP>
-__device__ __forceinline__ void flux_pass(Resident<NZ, CAP>& r, const WorkAddr& f) {
+template <int NZ, class CAP>
+__device__ __forceinline__ void flux_pass(const Resident<NZ, CAP>& r, const WorkAddr& f) {
     using PK = typename Pack<NZ>::T;
     constexpr int n = Pack<NZ>::n;
-    constexpr uint32_t all = (1u << NZ) - 1;
     const int n1 = r.cnt & 15, n2 = r.cnt >> 4 & 15, na = r.cnt >> 8 & 15;
 #pragma unroll
     for (int i = 0; i < CAP::F1; ++i)
         if (i < n1) {
             PK y[n], fl[n];
-            if (EVERY) {
-                rates_of<NZ>(f, i, all, r.k1[i]);
-                st_zones<NZ>(f.V + 4 * ldu(f.p0 + i * f.cst), r.k1[i]);
-            }
             ld_zones<NZ>(lo16<4>(r.f1[i], f.Y), y);
 #pragma unroll
             for (int q = 0; q < n; ++q) fl[q] = pmul(r.k1[i][q], y[q]);
@@ -327,7 +329,6 @@ __device__ __forceinline__ void flux_pass(Resident<NZ, CAP>& r, const WorkAddr& 
     for (int i = 0; i < CAP::F2; ++i)
         if (i < n2) {
             PK ya[n], yb[n], fl[n], a0[n], a1[n];
-            if (EVERY) rates_of<NZ>(f, CAP::F1 + i, all, r.k2[i]);
             ld_zones<NZ>(lo16<4>(r.f2[i][0], f.Y), ya);
             ld_zones<NZ>(hi16<4>(r.f2[i][0], f.Y), yb);
 #pragma unroll
@@ -347,7 +348,6 @@ __device__ __forceinline__ void flux_pass(Resident<NZ, CAP>& r, const WorkAddr& 
         if (i < na) {
             const uint32_t nr = r.fa[i][3] >> 16;
             PK ya[n], yb[n], yc[n], fl[n], a0[n], a1[n], a2[n];
-            if (EVERY) rates_of<NZ>(f, CAP::F1 + CAP::F2 + i, all, r.ka[i]);
             ld_zones<NZ>(lo16<4>(r.fa[i][0], f.Y), ya);
             ld_zones<NZ>(hi16<4>(r.fa[i][0], f.Y), yb);
             ld_zones<NZ>(lo16<4>(r.fa[i][1], f.Y), yc);
@@ -581,17 +581,25 @@ __device__ __forceinline__ void butterfly(const typename Pack<NZ>::T (&ch)[Pack<
 }
 
 // ---------------------------------------------------------------------------
-// warp 0, a zone's lanes: what the next decision needs and does not depend on
-// its outcome (FP64; runs beside the update)
+// A zone's lanes: what the next decision needs and does not depend on its outcome.
+// In three stages, so that a single warp can put other work between an FP64
+// operation and the use of its result.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void prepare_attempt(Scal& S, const PlanDev& P) {
-    const double ts = S.t + (double)S.h;
-    S.tf = __double2float_rn(ts);
+__device__ __forceinline__ void prepare_1(Scal& S) { S.ts = S.t + (double)S.h; }
+__device__ __forceinline__ void prepare_2(Scal& S) {
+    S.tf = __double2float_rn(S.ts);
+    S.ta = S.clip ? S.te : S.ts;
+    S.rem_d = S.te - S.ta;
+}
+__device__ __forceinline__ void prepare_3(Scal& S, const PlanDev& P) {
     S.u = S.cst ? 0.f : __fmul_rn(S.tf, S.us);
-    S.refresh = S.live && !(fabsf(S.u - S.ur) <= P.u_tol);
-    S.ta = S.clip ? S.te : ts;
-    S.rem_acc = (float)(S.te - S.ta);
+    S.rem_acc = (float)S.rem_d;
     S.last = S.clip || !(S.ta < S.te);
+    // the cached rates serve while no rate moves by a quarter ulp; without a cache
+    // (large networks: every pass takes the rates at its own u) while every factor
+    // 2^(-c u) is 1, as it is at the cached rates' u
+    S.refresh = S.live && (P.rate_cache ? !(fabsf(S.u - S.ur) <= P.u_tol)
+                                        : !(fabsf(S.u) <= P.u_one && fabsf(S.ur) <= P.u_one));
 }
 
 // accept or reject the attempt and set up the next one: decide_mixed's rules
@@ -902,7 +910,7 @@ __device__ __forceinline__ void predict_species(uint32_t row, uint32_t Yi, const
 // beside the update and decides beside the flux pass.  Barriers per attempt:
 // after the gather, the update and the decision.
 // ---------------------------------------------------------------------------
-template <int NZ, bool QSS, bool EVERY, class CAP>
+template <int NZ, bool QSS, class CAP>
 __device__ __forceinline__ void run_workers(const PlanDev& P, const OptsDev& O, const SlotBase g, SlotCtl& C, const int tid,
                                             const SlotSync<false> gs) {
     using PK = typename Pack<NZ>::T;
@@ -912,99 +920,94 @@ __device__ __forceinline__ void run_workers(const PlanDev& P, const OptsDev& O, 
     const uint32_t Yi = g.gb + P.sl.off_Y + at<NZ>(tid), row = g.gb + P.sl.off_Fk + 8 * NZ * tid,
                    Fk = g.gb + P.sl.off_Fk, ctl = g.gb + P.sl.off_ctl;
     const float A = mine ? ((const float*)(P.blob + P.tl.off_A))[tid] : 0.f;
-    const WorkAddr f = work_addr<NZ>(P, g, tid, Tw);
+    const WorkAddr f = work_addr(P, g);
     Resident<NZ, CAP> res;
     res.load(P, tid, Tw);
-    PK yh[n], yl[n], nh[n], nl[n];
+    PK yh[n], yl[n];
 #pragma unroll
     for (int q = 0; q < n; ++q) {
         pall(yh[q], 0.f);
         pall(yl[q], 0.f);
-        pall(nh[q], 0.f);
-        pall(nl[q], 0.f);
     }
-    uint32_t done = (1u << NZ) - 1, need = 0;  // at first every slot is to be filled
+    uint32_t done = (1u << NZ) - 1;  // at first every slot is to be filled
     for (;;) {
-        uint32_t rm = 0;
-        if (done) {
-            if (mine)
+        // ---- a zone ended: once per zone ----
+        if (mine)
 #pragma unroll
-                for (int z = 0; z < NZ; ++z)
-                    if (done >> z & 1) {
-                        sts(row + 4 * z, zget<NZ>(yh, z));
-                        sts(row + 4 * (NZ + z), zget<NZ>(yl, z));
-                    }
-            Scal none;
-            change_zones<NZ, false>(P, O, g, C, tid, P.T, done, none);
-            if (!C.live) break;
-            if (mine)
+            for (int z = 0; z < NZ; ++z)
+                if (done >> z & 1) {
+                    sts(row + 4 * z, zget<NZ>(yh, z));
+                    sts(row + 4 * (NZ + z), zget<NZ>(yl, z));
+                }
+        Scal none;
+        change_zones<NZ, false>(P, O, g, C, tid, P.T, done, none);
+        if (!C.live) break;
+        if (mine)
 #pragma unroll
-                for (int z = 0; z < NZ; ++z)
-                    if (done >> z & 1) {
-                        zset<NZ>(yh, z, lds(row + 4 * z));
-                        zset<NZ>(yl, z, lds(row + 4 * (NZ + z)));
-                    }
-            rm = C.fresh;
-            need |= rm;
+            for (int z = 0; z < NZ; ++z)
+                if (done >> z & 1) {
+                    zset<NZ>(yh, z, lds(row + 4 * z));
+                    zset<NZ>(yl, z, lds(row + 4 * (NZ + z)));
+                }
+        const uint32_t fresh = C.fresh;
+        if (fresh) {
+            // (a) and (b) of the new zones' first states (the other zones' values come
+            // out as they were, and are not stored)
+            refresh_rates<NZ>(P, g, tid, Tw, res, f, fresh);
+            flux_pass<NZ>(res, f);
+            gs.sync();
+            gather_pass<NZ>(res, f.V, Fk, fresh);
+            gs.sync();
         }
-        // the loop below leaves after an update's flux pass; new zones enter it at
-        // their first one (the other zones' values come out as they were)
-        bool first = rm != 0;
-        for (;;) {
-            if (!first) {
-                // ---- (b) the gathers of the states just reached ----
-                if (need) {
-                    gather_pass<NZ>(res, f.V, Fk, need);
-                    gs.sync();
-                }
-                PK h[n];
+        // ---- steps, until a zone ends ----
+        do {
+            PK h[n], nh[n], nl[n];
 #pragma unroll
-                for (int q = 0; q < n; ++q) ldp(ctl + (int)sizeof(PK) * q, h[q]);
-                if (QSS) {  // the predicted state's (F+, k)
-                    if (mine) predict_species<NZ>(row, Yi, yh, h);
-                    gs.sync();
-                    const uint32_t pm = C.rmask;
-                    if (!EVERY && pm) refresh_rates<NZ>(res, f, pm);
-                    flux_pass<NZ, EVERY>(res, f);
-                    gs.sync();
-                    gather_pass<NZ>(res, f.V, g.gb + P.sl.off_Fk2, (1u << NZ) - 1);
-                    gs.sync();
-                }
-                // ---- (d) update and error measures ----
-                if (w < nsw) {
-                    float ch, cl;
-                    uint32_t rb;
-                    update_warp<NZ, QSS>(O, mine, row, g.gb + P.sl.off_Fk2 + 8 * NZ * tid, Yi, A, lane, yh, yl, h, nh, nl,
-                                         ch, cl, rb);
-                    if ((lane & (LZ - 1)) == 0)
-                        asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %3};" ::"r"(g.gb + P.sl.off_red +
-                                                                                      16 * (w * NZ + lane / LZ)),
-                                     "f"(ch), "f"(cl), "f"(__uint_as_float(rb))
-                                     : "memory");
-                }
+            for (int q = 0; q < n; ++q) ldp(ctl + (int)sizeof(PK) * q, h[q]);
+            if (QSS) {  // the predicted state's (F+, k)
+                if (mine) predict_species<NZ>(row, Yi, yh, h);
                 gs.sync();
-                rm = QSS ? 0u : ldu(ctl + 24);  // SlotCtl::rmask
+                const uint32_t pm = C.rmask;
+                if (pm) refresh_rates<NZ>(P, g, tid, Tw, res, f, pm);
+                flux_pass<NZ>(res, f);
+                gs.sync();
+                gather_pass<NZ>(res, f.V, g.gb + P.sl.off_Fk2, (1u << NZ) - 1);
+                gs.sync();
             }
+            // ---- (d) update and error measures ----
+            if (w < nsw) {
+                float ch, cl;
+                uint32_t rb;
+                update_warp<NZ, QSS>(O, mine, row, g.gb + P.sl.off_Fk2 + 8 * NZ * tid, Yi, A, lane, yh, yl, h, nh, nl, ch,
+                                     cl, rb);
+                if ((lane & (LZ - 1)) == 0)
+                    asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %3};" ::"r"(g.gb + P.sl.off_red +
+                                                                                  16 * (w * NZ + lane / LZ)),
+                                 "f"(ch), "f"(cl), "f"(__uint_as_float(rb))
+                                 : "memory");
+            }
+            gs.sync();
             // ---- (a) for the candidate states, as the accepted zones' next attempts
             // need it, while the control warp decides ----
-            if (!EVERY && rm) refresh_rates<NZ>(res, f, rm);
-            flux_pass<NZ, EVERY>(res, f);
+            const uint32_t rm = QSS ? 0u : ldu(ctl + 24);  // SlotCtl::rmask
+            if (rm) refresh_rates<NZ>(P, g, tid, Tw, res, f, rm);
+            flux_pass<NZ>(res, f);
             gs.sync();
-            if (first) {
-                first = false;
-                continue;
-            }
+            // ---- (b) the gathers, stored for the accepted zones ----
             const uint2 ad = ldu2(ctl + 16);  // SlotCtl::acc, done
+            done = ad.y;
 #pragma unroll
             for (int z = 0; z < NZ; ++z)
                 if (ad.x >> z & 1) {
                     zset<NZ>(yh, z, zget<NZ>(nh, z));
                     zset<NZ>(yl, z, zget<NZ>(nl, z));
                 }
-            done = ad.y;
-            need = ad.x & ~ad.y;
-            if (done) break;
-        }
+            // (rejected zones repeat their attempts with the (F+, k) they have)
+            if (ad.x) {
+                gather_pass<NZ>(res, f.V, Fk, ad.x & ~ad.y);
+                gs.sync();
+            }
+        } while (!done);
     }
 }
 
@@ -1016,23 +1019,25 @@ __device__ __forceinline__ void run_control(const PlanDev& P, const OptsDev& O, 
     const uint32_t red = g.gb + P.sl.off_red + 16 * cz;
     const bool head = lane == cz * LZ;
     Scal S{};
-    uint32_t done = (1u << NZ) - 1, need = 0;
+    uint32_t done = (1u << NZ) - 1;
     for (;;) {
         if (done) {
             Scal X = S;  // a copy, so that S itself stays in registers
             change_zones<NZ, false>(P, O, g, C, tid, P.T, done, X);
             S = X;
             if (!C.live) break;
-            const uint32_t fresh = C.fresh;
-            if (fresh) gs.sync();
-            need |= fresh;
+            if (C.fresh) {  // the new zones' flux pass and gathers
+                gs.sync();
+                gs.sync();
+            }
         }
         // what the decision needs and does not depend on its outcome; the flux pass
         // refreshes the cached rates whatever the outcome
-        prepare_attempt(S, P);
+        prepare_1(S);
+        prepare_2(S);
+        prepare_3(S, P);
         const uint32_t rm = zone_bits<NZ>(S.refresh);
         if (S.refresh) S.ur = S.u;
-        if (need) gs.sync();
         if (head) C.u[cz] = S.u;
         if (lane == 0) C.rmask = rm;
         if (QSS) {
@@ -1054,7 +1059,7 @@ __device__ __forceinline__ void run_control(const PlanDev& P, const OptsDev& O, 
         }
         gs.sync();
         done = dm;
-        need = am & ~dm;
+        if (am) gs.sync();  // the workers' gather
     }
 }
 
@@ -1062,7 +1067,7 @@ __device__ __forceinline__ void run_control(const PlanDev& P, const OptsDev& O, 
 // A group of one warp (small networks): everything in turn, the scalars in
 // registers, a zone's in its share of the lanes.
 // ---------------------------------------------------------------------------
-template <int NZ, bool QSS, bool EVERY, class CAP>
+template <int NZ, bool QSS, class CAP>
 __device__ __forceinline__ void run_warp(const PlanDev& P, const OptsDev& O, const SlotBase g, SlotCtl& C, const int lane) {
     using PK = typename Pack<NZ>::T;
     constexpr int n = Pack<NZ>::n, LZ = 32 / NZ;
@@ -1072,7 +1077,7 @@ __device__ __forceinline__ void run_warp(const PlanDev& P, const OptsDev& O, con
     const uint32_t Yi = g.gb + P.sl.off_Y + at<NZ>(lane), row = g.gb + P.sl.off_Fk + 8 * NZ * lane,
                    Fk = g.gb + P.sl.off_Fk;
     const float A = mine ? ((const float*)(P.blob + P.tl.off_A))[lane] : 0.f;
-    const WorkAddr f = work_addr<NZ>(P, g, lane, 32);
+    const WorkAddr f = work_addr(P, g);
     Resident<NZ, CAP> res;
     res.load(P, lane, 32);
     PK yh[n], yl[n];
@@ -1107,21 +1112,28 @@ __device__ __forceinline__ void run_warp(const PlanDev& P, const OptsDev& O, con
             rm = C.fresh;
             need |= rm;
         }
+        // (a) of the states just reached: only they refresh their cached rates (a new
+        // zone computes them, at the u set with it); beside it the FP64 work of the
+        // next attempt
         if (need) {
-            // (a) of the states just reached: only they refresh their cached rates
-            // (a new zone computes them, at the u set with it)
             const bool go = (need & ~rm) >> cz & 1;
             rm |= zone_bits<NZ>(go && S.refresh);
             if (go && S.refresh) S.ur = S.u;
             if (go && lane == cz * LZ) C.u[cz] = S.u;
             gs.sync();
-            if (!EVERY && rm) refresh_rates<NZ>(res, f, rm);
-            flux_pass<NZ, EVERY>(res, f);
+        }
+        prepare_1(S);
+        if (need) {
+            if (rm) refresh_rates<NZ>(P, g, lane, 32, res, f, rm);
+            flux_pass<NZ>(res, f);
             gs.sync();
+        }
+        prepare_2(S);
+        if (need) {
             gather_pass<NZ>(res, f.V, Fk, need);
             gs.sync();
         }
-        prepare_attempt(S, P);
+        prepare_3(S, P);
         PK h[n], nh[n], nl[n];
 #pragma unroll
         for (int z = 0; z < NZ; ++z) zset<NZ>(h, z, __shfl_sync(0xffffffffu, S.h, z * LZ));
@@ -1132,8 +1144,8 @@ __device__ __forceinline__ void run_warp(const PlanDev& P, const OptsDev& O, con
             S.refresh = false;
             if (lane == cz * LZ) C.u[cz] = S.u;
             gs.sync();
-            if (!EVERY && pm) refresh_rates<NZ>(res, f, pm);
-            flux_pass<NZ, EVERY>(res, f);
+            if (pm) refresh_rates<NZ>(P, g, lane, 32, res, f, pm);
+            flux_pass<NZ>(res, f);
             gs.sync();
             gather_pass<NZ>(res, f.V, g.gb + P.sl.off_Fk2, (1u << NZ) - 1);
             gs.sync();
@@ -1162,13 +1174,13 @@ template <int A1, int A2, int A3, int A4, int A5> struct Cap {
 #define CAP_OF(k) Cap<kSlotCaps[k].f1, kSlotCaps[k].f2, kSlotCaps[k].fa, kSlotCaps[k].ga, kSlotCaps[k].gb>
 
 // one plan's groups
-template <int NZ, bool QSS, bool EVERY, int CK>
+template <int NZ, bool QSS, int CK>
 __device__ __forceinline__ void run_plan(const PlanDev& P, const OptsDev& O, const SlotBase g, SlotCtl& C, int gr, int tid) {
     if (CK == kCapWarp) {
-        run_warp<NZ, QSS, EVERY, CAP_OF(CK)>(P, O, g, C, tid);
+        run_warp<NZ, QSS, CAP_OF(CK)>(P, O, g, C, tid);
     } else {
         const SlotSync<false> gs{1 + gr, P.T};
-        if (tid < P.T - 32) run_workers<NZ, QSS, EVERY, CAP_OF(CK)>(P, O, g, C, tid, gs);
+        if (tid < P.T - 32) run_workers<NZ, QSS, CAP_OF(CK)>(P, O, g, C, tid, gs);
         else run_control<NZ, QSS>(P, O, g, C, tid, gs);
     }
 }
@@ -1213,11 +1225,11 @@ __global__ void __launch_bounds__(kSlotThreads, 1) slots_kernel(const __grid_con
             }
             // (change_zones begins with a barrier)
             if constexpr (ONE) {
-                run_plan<NZ, QSS, CK == kCapEvery, CK>(P, lp.o, g, C, gr, tid);
+                run_plan<NZ, QSS, CK>(P, lp.o, g, C, gr, tid);
             } else {
-                if (P.cap == kCapWarp) run_plan<NZ, QSS, false, kCapWarp>(P, lp.o, g, C, gr, tid);
-                else if (P.cap == kCapEvery) run_plan<NZ, QSS, true, kCapEvery>(P, lp.o, g, C, gr, tid);
-                else run_plan<NZ, QSS, false, kCapGroup>(P, lp.o, g, C, gr, tid);
+                if (P.cap == kCapWarp) run_plan<NZ, QSS, kCapWarp>(P, lp.o, g, C, gr, tid);
+                else if (P.cap == kCapWide) run_plan<NZ, QSS, kCapWide>(P, lp.o, g, C, gr, tid);
+                else run_plan<NZ, QSS, kCapGroup>(P, lp.o, g, C, gr, tid);
             }
         }
         __syncthreads();
@@ -1229,7 +1241,7 @@ template <int NZ, bool QSS> SlotsFn slots_fn(int cap) {
     switch (cap) {
         case kCapWarp: return slots_kernel<NZ, QSS, kCapWarp>;
         case kCapGroup: return slots_kernel<NZ, QSS, kCapGroup>;
-        case kCapEvery: return slots_kernel<NZ, QSS, kCapEvery>;
+        case kCapWide: return slots_kernel<NZ, QSS, kCapWide>;
         default: return slots_kernel<NZ, QSS, kCapMany>;
     }
 }
