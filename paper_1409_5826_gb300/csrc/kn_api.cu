@@ -5,6 +5,7 @@
 #include <cub/device/device_radix_sort.cuh>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -13,6 +14,7 @@
 #include <map>
 #include <memory>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include "kn_host.h"
@@ -61,6 +63,50 @@ static kn_status get_tables(kn_network* n, int prec, int Q, Tables** out) {
         it = n->tables.emplace(key, std::move(T)).first;
     }
     *out = &it->second;
+    return KN_OK;
+}
+
+// The tables of every group size G0, G0 + 32, .. G1, the missing ones built side by
+// side: a default launch looks at up to 12 of them (5 ms each for 150/1604).
+static kn_status build_tables_range(kn_network* n, int prec, int G0, int G1) {
+    struct Job {
+        int G;
+        std::vector<unsigned char> blob;
+        Tables T;
+        kn_status s;
+        std::string msg;
+    };
+    std::vector<Job> jobs;
+    for (int G = G0; G <= G1; G += 32)
+        if (!n->tables.count({prec, G})) jobs.push_back({G, {}, {}, KN_OK, {}});
+    if (jobs.size() < 2) return KN_OK;  // get_tables builds it
+    std::atomic<size_t> next{0};
+    auto work = [&]() {
+        for (size_t i; (i = next.fetch_add(1)) < jobs.size();) {
+            Job& j = jobs[i];
+            try {
+                j.s = build_tables_host(n, prec, j.G, j.blob, j.T);
+                if (j.s != KN_OK) j.msg = last_error();  // the message is this thread's
+            } catch (const std::exception&) {
+                j.s = KN_ERR_NOMEM;
+            }
+        }
+    };
+    std::vector<std::thread> pool;
+    const size_t threads = std::min<size_t>(jobs.size(), std::max(1u, std::thread::hardware_concurrency()));
+    try {
+        while (pool.size() + 1 < threads) pool.emplace_back(work);
+    } catch (const std::exception&) {  // no more threads: the ones there are do the work
+    }
+    work();
+    for (auto& t : pool) t.join();
+    for (Job& j : jobs) {
+        if (j.s != KN_OK) return fail(j.s, "%s", j.msg.c_str());
+        j.T.blob.reset(new DevBuf());
+        KN_CUDA(j.T.blob->ensure(j.blob.size()));
+        KN_CUDA(cudaMemcpy(j.T.blob->p, j.blob.data(), j.blob.size(), cudaMemcpyHostToDevice));
+        n->tables.emplace(std::make_pair(prec, j.G), std::move(j.T));
+    }
     return KN_OK;
 }
 
@@ -580,6 +626,7 @@ static kn_status prepare_launch(kn_network* const* nets, int n_nets, const kn_op
             const int g1 = o->threads_per_zone ? o->threads_per_zone : 512;
             const bool small = g0 == 32 || prec != kPrecMixed;
             constexpr int kTargetGroups = 5;
+            if ((s = build_tables_range(n, prec, g0, g1)) != KN_OK) return s;
             for (int G = g0; G <= g1; G += 32) {
                 Tables* tb;
                 if ((s = get_tables(n, prec, G, &tb)) != KN_OK) return s;
