@@ -561,6 +561,11 @@ static void set_guard_band(OptsDev& D, const kn_opts* o) {
     D.ga32 = (float)(o->safety * o->eps_r);
     D.gb32 = (float)(o->safety * o->eps_c);
     D.grow32 = (float)o->grow_max;
+    // the FP64 form's approximate test reads ratios from 2^-100 to 2^99 and clamps the
+    // growth terms' denominators at 1e-30: the limits have to lie well inside
+    D.fast64 = o->y_min >= 1e-250 && o->eps_r >= 1e-20 && o->eps_r <= 1e20 && o->eps_c <= 1e20 &&
+               o->safety * o->eps_r >= 1e-25 && o->safety * o->eps_c >= 1e-25 &&
+               o->grow_max < 1e29 * o->safety * std::min(o->eps_r, o->eps_c);
     D.shrink32 = (float)o->shrink;
     D.dt_min32 = (float)o->dt_min_frac;
     D.band_lo32 = (float)(1.0 - band);

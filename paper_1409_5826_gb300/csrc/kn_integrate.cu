@@ -55,6 +55,38 @@ __device__ __forceinline__ double exp_neg_small(double x, int degree) {
     return fma(x, p, 1.0);
 }
 
+// FP64 rate factors in integers.  On this chip a warp's FP64 instruction takes the
+// SM's FP64 pipe for 20 cycles and an integer one costs a fortieth of that, so the
+// three FP64 operations of exp_neg_small(x, 2), x = fl(c s), are replaced by an
+// integer evaluation of the same value: below 1 the factor is 1 - m 2^-53 with the
+// integer m nearest to W = 2^53 x (1 - x/2).  W is formed in fixed point, 22 fraction
+// bits, with an error of less than 12 of their units (the roundings of x and of
+// 1 - x/2 included: at most 3), and a W within 64 units of a rounding boundary is
+// left to the FP64 operations.  (608 zones of 150/1604: 276 ms with the FP64 factors
+// and products in the accept test, 157 ms with this and ratio_approx.)
+//
+// s in fixed point: 2^82 s, for 0 <= s < 2^-20
+__device__ __forceinline__ unsigned long long factor_scale(double s) {
+    return __double2ull_rn(s * 4835703278458516698824704.0);
+}
+// the factor for 2^53 c s < 2^32; ok = false: W too near a boundary, or c outside [2^-20, 128)
+__device__ __forceinline__ double factor_small(double c, unsigned long long sf, bool& ok) {
+    const unsigned int ch = (unsigned int)__double2hiint(c), cl = (unsigned int)__double2loint(c);
+    const int sh = 1029 - (int)(ch >> 20);  // 6 - (c's exponent)
+    // c's mantissa with its top bit at 63, times sf: the high 64 bits (the product of
+    // the low words left out: at most two units too small)
+    const unsigned int ah = __funnelshift_l(cl, (ch & 0xfffffu) | 0x100000u, 11), al = cl << 11;
+    const unsigned int sh_ = (unsigned int)(sf >> 32), sl = (unsigned int)sf;
+    const unsigned long long hi = (unsigned long long)ah * sh_ + __umulhi(ah, sl) + __umulhi(al, sh_);
+    const unsigned long long X = hi >> (sh & 63);  // 2^53 c s with 22 fraction bits
+    const unsigned int xi = (unsigned int)(X >> 22);
+    const unsigned long long W = X - __umulhi(xi, xi);
+    const unsigned int f = (unsigned int)W & 0x3fffffu;
+    ok = (unsigned int)sh <= 26u && f - (0x200000u - 64u) > 128u;
+    const unsigned long long m = (W + 0x200000ull) >> 22;
+    return __longlong_as_double(0x3ff0000000000000ll - (long long)m);
+}
+
 // Kahan-compensated FP32 sum (the gathers of the mixed form with the FP64 update).
 struct AccKahan {
     float s, c;  // sum and (negated) lost low part: value = s - c
@@ -240,6 +272,21 @@ __device__ __forceinline__ void qss_predict_mixed(const PlanDev& P, const GroupP
     }
 }
 
+// |d| / m for finite doubles and m > 2^-900, to within 2^-20, without an FP64
+// instruction: the quotient of the leading 24 bits, scaled.  Below 2^-100 it is 0,
+// from 2^101 on it is at least 2^99.
+__device__ __forceinline__ float ratio_approx(double d, double m) {
+    const unsigned int dh = (unsigned int)__double2hiint(d) & 0x7fffffffu, mh = (unsigned int)__double2hiint(m);
+    const float a = __uint_as_float(0x3f800000u | (dh & 0xfffffu) << 3 | (unsigned int)__double2loint(d) >> 29);
+    const float b = __uint_as_float(0x3f800000u | (mh & 0xfffffu) << 3 | (unsigned int)__double2loint(m) >> 29);
+    const int e = (int)(dh >> 20) - (int)(mh >> 20);
+    const float q = __fdividef(a, b);
+    return e < -100 ? 0.f : __int_as_float(__float_as_int(q) + (min(e, 100) << 23));
+}
+
+// x >= y for doubles x >= 0 and y > 0 (a NaN x counts as larger): their bits order as integers
+__device__ __forceinline__ bool ge_bits(double x, double y) { return __double_as_longlong(x) >= __double_as_longlong(y); }
+
 // (d) the update with step h from buffer cur into nxt, and each warp's share
 // of the error measures (no barrier inside).  FP64 form: every step in FP64,
 // in the order of the definitions.  QSS = false: the kappa-switched update
@@ -247,7 +294,50 @@ __device__ __forceinline__ void qss_predict_mixed(const PlanDev& P, const GroupP
 // state's (F+, k) and the predicted state's (F+p, kp) in Fk2:
 //   kbar = (k + kp)/2, a = alpha(kbar h),
 //   Y' = Y + h (a F+p + (1 - a) F+ - kbar Y) / (1 + a kbar h).
-template <bool QSS>
+// EXACT: the largest relative change as a fraction bn / bd, compared by products in
+// FP64 (three FP64 operations a species and three a butterfly level).  Otherwise the
+// warp leaves an approximate largest ratio and the species that has it (-1: others
+// come within 2^-18 of it), from which the decision forms the fraction if it needs
+// it; where it cannot, exact_ratios does the EXACT reduction afterwards.
+__device__ __forceinline__ void ratio_reduce(const GroupPtrs& g, int lane, double bn, double bd) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        const double on = __shfl_xor_sync(0xffffffffu, bn, off);
+        const double od = __shfl_xor_sync(0xffffffffu, bd, off);
+        if (on * bd > bn * od) {
+            bn = on;
+            bd = od;
+        }
+    }
+    if ((lane & 31) == 0) {
+        g.red_n[lane >> 5] = bn;
+        g.red_d[lane >> 5] = bd;
+    }
+}
+
+// the larger of the fractions bn / bd and |d| / max(y, yn), the latter if it is tested
+__device__ __forceinline__ void ratio_max(double y, double yn, double d, double ymin, double& bn, double& bd) {
+    if ((y > yn ? y : yn) > ymin) {
+        const double m = y > yn ? y : yn;
+        const double ad = fabs(d);
+        if (ad * bd > bn * m) {
+            bn = ad;
+            bd = m;
+        }
+    }
+}
+
+// the EXACT reduction of an attempt already taken, from the two states
+__device__ __forceinline__ void exact_ratios(const PlanDev& P, const OptsDev& O, const GroupPtrs& g, int lane, int cur) {
+    if ((lane & ~31) >= P.N) return;
+    const double* Yc = g.Y64 + cur * (P.N + 1);
+    const double* Yn = g.Y64 + (cur ^ 1) * (P.N + 1);
+    double bn = 0.0, bd = 1.0;
+    for (int i = lane; i < P.N; i += P.G) ratio_max(Yc[i], Yn[i], Yn[i] - Yc[i], O.y_min, bn, bd);
+    ratio_reduce(g, lane, bn, bd);
+}
+
+template <bool QSS, bool EXACT>
 __device__ __forceinline__ void update_reduce_fp64(const PlanDev& P, const OptsDev& O, const GroupPtrs& g, int lane,
                                                    int cur, double h, int z) {
     if ((lane & ~31) >= P.N) return;  // a warp without species
@@ -259,6 +349,8 @@ __device__ __forceinline__ void update_reduce_fp64(const PlanDev& P, const OptsD
     double* Yn64 = g.Y64 + (cur ^ 1) * NP1;
     const double kappa = O.kappa, ymin = O.y_min;
     double csum = 0.0, bn = 0.0, bd = 1.0;
+    float rmax = 0.f;
+    int who = -1;
     for (int i = lane; i < N; i += G) {
         const double y = Yc[i], fp = Fk[2 * i], kk = Fk[2 * i + 1];
         double yn;
@@ -266,17 +358,20 @@ __device__ __forceinline__ void update_reduce_fp64(const PlanDev& P, const OptsD
             yn = qss_correct1(y, Fk2[2 * i], fp, 0.5 * (kk + Fk2[2 * i + 1]), h);
         } else {
             const double kdt = kk * h;
-            yn = (kdt >= kappa) ? (y + h * fp) / (1.0 + kdt) : y + h * (fp - kk * y);
+            yn = ge_bits(kdt, kappa) ? (y + h * fp) / (1.0 + kdt) : y + h * (fp - kk * y);
         }
         Yn64[i] = yn;
         const double d = yn - y;
         csum = fma(A[i], d, csum);
-        if ((y > yn ? y : yn) > ymin) {
-            const double m = y > yn ? y : yn;
-            const double ad = fabs(d);
-            if (ad * bd > bn * m) {
-                bn = ad;
-                bd = m;
+        if (EXACT) {
+            ratio_max(y, yn, d, ymin, bn, bd);
+        } else {
+            // y >= 0, so the larger of y and yn has the larger bits
+            const double m = __double_as_longlong(y) > __double_as_longlong(yn) ? y : yn;
+            if (__double_as_longlong(m) > __double_as_longlong(ymin)) {
+                const float r = ratio_approx(d, m);
+                if (r >= rmax * (1.f - 3.8146972656e-06f)) who = r * (1.f - 3.8146972656e-06f) > rmax ? i : -1;
+                rmax = fmaxf(rmax, r);
             }
         }
         if (O.probe) {
@@ -286,20 +381,18 @@ __device__ __forceinline__ void update_reduce_fp64(const PlanDev& P, const OptsD
         }
     }
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        csum += __shfl_xor_sync(0xffffffffu, csum, off);
-        const double on = __shfl_xor_sync(0xffffffffu, bn, off);
-        const double od = __shfl_xor_sync(0xffffffffu, bd, off);
-        if (on * bd > bn * od) {
-            bn = on;
-            bd = od;
+    for (int off = 16; off > 0; off >>= 1) csum += __shfl_xor_sync(0xffffffffu, csum, off);
+    if ((lane & 31) == 0) g.red_c[lane >> 5] = csum;
+    if (EXACT) {
+        ratio_reduce(g, lane, bn, bd);
+    } else {
+        const float R = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(rmax)));
+        const unsigned int near = __ballot_sync(0xffffffffu, rmax >= R * (1.f - 3.8146972656e-06f));
+        who = __shfl_sync(0xffffffffu, who, __ffs(near) - 1);
+        if ((lane & 31) == 0) {
+            g.red_r[lane >> 5] = R;
+            g.red_f[lane >> 5] = __popc(near) == 1 ? who : -1;
         }
-    }
-    if ((lane & 31) == 0) {
-        const int w = lane >> 5;
-        g.red_c[w] = csum;
-        g.red_n[w] = bn;
-        g.red_d[w] = bd;
     }
 }
 
@@ -506,7 +599,7 @@ __device__ __forceinline__ void update_reduce_mixed64(const PlanDev& P, const Op
 
 // h: the step (FP64 forms); h32: the same step in FP32 (the mixed form's update);
 // QSS: the alpha-QSS corrector instead of Eq. 3 (FP64 form)
-template <int PREC, bool QSS = false>
+template <int PREC, bool QSS = false, bool EXACT = true>
 __device__ __forceinline__ void update_reduce(const PlanDev& P, const OptsDev& O, const GroupPtrs& g, int lane,
                                               int cur, double h, float h32, int z) {
     if (PREC == kPrecMixed)
@@ -514,7 +607,7 @@ __device__ __forceinline__ void update_reduce(const PlanDev& P, const OptsDev& O
     else if (PREC == kPrecMixed64)
         update_reduce_mixed64(P, O, g, lane, cur, h, z);
     else
-        update_reduce_fp64<QSS>(P, O, g, lane, cur, h, z);
+        update_reduce_fp64<QSS, EXACT>(P, O, g, lane, cur, h, z);
 }
 
 // lane 0, after the barrier that follows update_reduce: combine the warps.
@@ -651,6 +744,95 @@ __device__ __forceinline__ void decide_mixed(GroupState& S, const PlanDev& P, co
         S.clipped = c;
         S.h32 = c ? rem_cur : dt;
     }
+}
+
+// lane 0, FP64 form, plain integration: the decision from the warps' conservation
+// sums and approximate largest ratios.  The exact fraction bn / bd of the largest
+// relative change, and its quotient, are formed only where they matter: the accept
+// test's outcome is clear unless the ratio lies within 2^-15 of eps_r, and only the
+// smallest term of the growth factor is divided out (a double division's latency is
+// 640 cycles, and the other lanes wait).  false: the fraction is needed and not known
+// (a near tie), and nothing has been decided.
+__device__ __forceinline__ bool decide_fp64(GroupState& S, const PlanDev& P, const OptsDev& O, const GroupPtrs& g,
+                                            int nxt, bool exact) {
+    const int nw = species_warps(P);
+    double cs = 0.0, bn = 0.0, bd = 1.0;
+    float R = 0.f, R2 = 0.f;
+    int who = -1;
+    for (int w = 0; w < nw; ++w) {
+        cs += g.red_c[w];
+        if (exact) {
+            const double on = g.red_n[w], od = g.red_d[w];
+            if (on * bd > bn * od) {
+                bn = on;
+                bd = od;
+            }
+        } else {
+            const float r = g.red_r[w];
+            R2 = fmaxf(R2, fminf(r, R));
+            if (r > R) {
+                R = r;
+                who = g.red_f[w];
+            }
+        }
+    }
+    if (exact) R = ratio_approx(bn, bd);
+    else if (R2 >= R * (1.f - 3.8146972656e-06f)) who = -1;
+    const int fin = isfinite(cs) ? 1 : 0;
+    const double cons = fabs(cs), h = S.h;
+    bool known = exact;
+    auto fraction = [&]() {
+        if (!known && who >= 0) {
+            const double y = g.Y64[S.cur * (P.N + 1) + who], yn = g.Y64[nxt * (P.N + 1) + who];
+            bn = fabs(yn - y);
+            bd = y > yn ? y : yn;
+            known = true;
+        }
+        return known;
+    };
+    bool pass = fin && cons <= O.eps_c;
+    if (pass) {
+        const float e = O.eps_r32;
+        if (R > e * (1.f + 3.0517578125e-05f)) pass = false;
+        else if (!(R < e * (1.f - 3.0517578125e-05f))) {
+            if (!fraction()) return false;
+            pass = bn <= O.eps_r * bd;
+        }
+    }
+    if (pass) {
+        // the proposal: h min(grow, safety eps_r / rel, safety eps_c / cons)
+        const float fa = __fdividef(O.ga32, fmaxf(R, 1e-30f)), fb = __fdividef(O.gb32, fmaxf((float)cons, 1e-30f));
+        double gfac = O.grow_max;
+        if (fa < 1.0001f * fminf(O.grow32, fb)) {
+            if (!fraction()) return false;
+            const double rel = bn / bd;
+            const double ga = O.safety * O.eps_r / (rel > 1e-300 ? rel : 1e-300);
+            if (ga < gfac) gfac = ga;
+        }
+        if (fb < 1.0001f * fminf(O.grow32, fa)) {
+            const double gb = O.safety * O.eps_c / (cons > 1e-300 ? cons : 1e-300);
+            if (gb < gfac) gfac = gb;
+        }
+        S.t = S.clipped ? S.t_end : S.t + h;
+        S.cur = nxt;
+        S.steps += 1;
+        S.nrej = 0;
+        S.rhs_valid = 0;
+        S.dt = h * gfac;
+    } else {
+        S.rejects += 1;
+        S.nrej += 1;
+        S.rhs_valid = 1;
+        S.dt = h * O.shrink;
+        if (S.nrej > O.max_reject) {
+            S.status = fin ? 4 : 3;  // MAX_REJECT : NONFINITE
+            S.done = 1;
+        } else if (S.dt < O.dt_min_frac * S.t) {
+            S.status = 2;  // DT_UNDERFLOW
+            S.done = 1;
+        }
+    }
+    return true;
 }
 
 // FP32 exponent histogram bin (4 octaves per bin, values below 2^-100 in bin 0)
@@ -868,11 +1050,19 @@ __device__ __forceinline__ void flux_pass(const PlanDev& P, const GroupPtrs& g, 
     const int pb1 = 2 * R - R1, pb2 = 3 * R - R1 - R12;  // bases of partial planes 1 and 2
     if (PREC == kPrecFP64) {
         const double* __restrict__ Yr = g.Y64 + buf * NP1;
+        // 2^53 c_max s < 2^32 (and s >= 0): the degree-2 factors in integers
+        const bool fixed = poly == 2 && P.cmax * s < 4.7e-7 && s < 9.5e-7;
+        const unsigned long long sf = fixed ? factor_scale(s) : 0;
 #pragma unroll 2
         for (int j = j0; j < R; j += stride) {
             const uint32_t rs = rspec[j];
             double k = (double)Kz[j];
-            if (poly == 2 || poly == 5)
+            bool ok = false;
+            double fac;
+            if (fixed) fac = factor_small((double)cexp[j], sf, ok);
+            if (ok)
+                k *= fac;
+            else if (poly == 2 || poly == 5)
                 k *= exp_neg_small((double)cexp[j] * s, poly);
             else if (poly == 9)
                 k *= exp(-(double)cexp[j] * s);
@@ -1300,12 +1490,31 @@ __device__ __forceinline__ void run_group(const PlanDev& P, const OptsDev& O, co
                 S.u_spec = S.constant ? 0.f : __fmul_rn(__double2float_rn(S.t + h_now), S.u_scale);
                 S.refresh_spec = !P.rate_cache || !(fabsf(S.u_spec - S.u_ref) <= P.u_tol);
             }
-            update_reduce<PREC, QSS>(P, O, g, lane, cur, h_now, PREC == kPrecMixed ? S.h32 : (float)h_now, z);
+            // FP64 form, plain integration: the approximate test (decide_fp64)
+            const bool fast = PREC == kPrecFP64 && !FEAT && O.fast64 && !O.probe && !O.replay_dt;
+            if (fast)
+                update_reduce<PREC, QSS, FEAT>(P, O, g, lane, cur, h_now, (float)h_now, z);
+            else
+                update_reduce<PREC, QSS>(P, O, g, lane, cur, h_now, PREC == kPrecMixed ? S.h32 : (float)h_now, z);
             gs.sync();
             if (spec && lane >= 32)
                 flux_pass<PREC>(P, g, lane - 32, G - 32, nxt, S.constant, 0.0, S.u_spec, 0, S.refresh_spec != 0);
             have_a = spec;
-            if (PREC == kPrecMixed && lane == 0 && !O.probe && !O.replay_dt) {
+            if (PREC == kPrecFP64 && fast) {
+                if (lane == 0) {
+                    S.found = decide_fp64(S, P, O, g, nxt, false);
+                    if (S.found) leader_prepare<PREC>(S, P, O);
+                }
+                gs.sync();
+                if (S.found) continue;
+                // a near tie of the largest ratios: reduced in full
+                exact_ratios(P, O, g, lane, cur);
+                gs.sync();
+                if (lane == 0) {
+                    decide_fp64(S, P, O, g, nxt, true);
+                    leader_prepare<PREC>(S, P, O);
+                }
+            } else if (PREC == kPrecMixed && lane == 0 && !O.probe && !O.replay_dt) {
                 decide_mixed<FEAT>(S, P, O, g, nxt, spec);
             } else if (lane == 0) {
                 if (spec && S.refresh_spec) S.u_ref = S.u_spec;  // the speculative pass refreshed Kc

@@ -227,6 +227,7 @@ struct OptsDev {
     float mlp_margin;  // the proposal uses e^(out - margin)
     // FP32 guard band of the mixed form's accept test (see update_reduce)
     float eps_r32, ymin_lo32, ymin_hi32, band_lo32, band_hi32, kappa32;
+    int fast64;  // FP64 form: the approximate test's range (1 = y_min and the limits lie inside)
     float eps_c32, ga32, gb32, grow32;  // mixed form: eps_c and the growth factor's terms in FP32
     float shrink32;                     // mixed form: the reject factor in FP32
     float dt_min32;                     // mixed form: dt_min_frac in FP32
