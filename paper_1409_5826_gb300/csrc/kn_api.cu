@@ -686,6 +686,8 @@ static kn_status prepare_launch(kn_network* const* nets, int n_nets, const kn_op
         P.cmax = n->cmax;
         P.u_tol = rate_cache_tol(n->cmax);
         P.u_one = one_tol(n->cmax);
+        P.one = 1.0;
+        P.neg_zero = -0.0;
         P.rate_cache = rate_cache_on(n, prec) ? 1 : 0;
         P.N = n->N;
         P.R = n->R;
@@ -981,6 +983,8 @@ kn_status noalloc_prepare(kn_network* n, const kn_opts* o, int32_t n_zones, cons
     Pd.R12 = n->R12;
     Pd.cmax = n->cmax;
     Pd.u_tol = rate_cache_tol(n->cmax);
+    Pd.one = 1.0;
+    Pd.neg_zero = -0.0;
     Pd.rate_cache = rate_cache_on(n, o->precision) ? 1 : 0;
     Pd.N = n->N;
     Pd.R = n->R;

@@ -55,37 +55,52 @@ __device__ __forceinline__ double exp_neg_small(double x, int degree) {
     return fma(x, p, 1.0);
 }
 
-// FP64 rate factors in integers.  On this chip a warp's FP64 instruction takes the
-// SM's FP64 pipe for 20 cycles and an integer one costs a fortieth of that, so the
-// three FP64 operations of exp_neg_small(x, 2), x = fl(c s), are replaced by an
-// integer evaluation of the same value: below 1 the factor is 1 - m 2^-53 with the
-// integer m nearest to W = 2^53 x (1 - x/2).  W is formed in fixed point, 22 fraction
-// bits, with an error of less than 12 of their units (the roundings of x and of
-// 1 - x/2 included: at most 3), and a W within 64 units of a rounding boundary is
-// left to the FP64 operations.  (608 zones of 150/1604: 276 ms with the FP64 factors
-// and products in the accept test, 157 ms with this and ratio_approx.)
+// FP64 rate factors in integers.  On this chip a warp's FP64 instruction takes an SM's
+// FP64 pipe for 16 cycles (fused) or 19 (a plain sum or product) and an integer one
+// costs a thirtieth of that, so the factor exp_neg_small(x, 2), x = fl(c s), is
+// evaluated in integers: it is 1 - m 2^-53 with the integer m nearest to
+// W = 2^53 x (1 - x/2).  W is formed in fixed point, 22 fraction bits, with an error
+// of less than 12 of their units (the roundings of x and of 1 - x/2 included: at most
+// 3), and a W within 64 units of a rounding boundary is left to the FP64 operations.
+// (608 zones of 150/1604: 276 ms with the FP64 factors and products in the accept
+// test, 157 ms with this and ratio_approx.)  Products in integers beside the pipe
+// (four 32-bit multiplications and some 25 other instructions) gained nothing: the
+// flux pass's latency grew by what the pipe was spared.
 //
 // s in fixed point: 2^82 s, for 0 <= s < 2^-20
 __device__ __forceinline__ unsigned long long factor_scale(double s) {
     return __double2ull_rn(s * 4835703278458516698824704.0);
 }
-// the factor for 2^53 c s < 2^32; ok = false: W too near a boundary, or c outside [2^-20, 128)
-__device__ __forceinline__ double factor_small(double c, unsigned long long sf, bool& ok) {
-    const unsigned int ch = (unsigned int)__double2hiint(c), cl = (unsigned int)__double2loint(c);
-    const int sh = 1029 - (int)(ch >> 20);  // 6 - (c's exponent)
-    // c's mantissa with its top bit at 63, times sf: the high 64 bits (the product of
-    // the low words left out: at most two units too small)
-    const unsigned int ah = __funnelshift_l(cl, (ch & 0xfffffu) | 0x100000u, 11), al = cl << 11;
-    const unsigned int sh_ = (unsigned int)(sf >> 32), sl = (unsigned int)sf;
-    const unsigned long long hi = (unsigned long long)ah * sh_ + __umulhi(ah, sl) + __umulhi(al, sh_);
-    const unsigned long long X = hi >> (sh & 63);  // 2^53 c s with 22 fraction bits
+
+// m, for 2^53 c s < 2^32; c = 0 gives 0; bad: W too near a boundary, or another c
+// outside [2^-20, 128)
+__device__ __forceinline__ unsigned int factor_small(double c, unsigned long long sf, bool& bad) {
+    const unsigned long long cb = (unsigned long long)__double_as_longlong(c);
+    const unsigned long long cm = (cb << 11) | 0x8000000000000000ull;
+    const int sh = 1029 - (int)(cb >> 52);  // 6 - (c's exponent)
+    // c's mantissa times sf: the high 64 bits (the product of the low words left out:
+    // at most two units too small)
+    const unsigned int ah = (unsigned int)(cm >> 32), al = (unsigned int)cm;
+    const unsigned int bh = (unsigned int)(sf >> 32), bl = (unsigned int)sf;
+    const unsigned long long hi = (unsigned long long)ah * bh + __umulhi(ah, bl) + __umulhi(al, bh);
+    const unsigned long long X = cb ? hi >> (sh & 63) : 0;  // 2^53 c s with 22 fraction bits
     const unsigned int xi = (unsigned int)(X >> 22);
     const unsigned long long W = X - __umulhi(xi, xi);
-    const unsigned int f = (unsigned int)W & 0x3fffffu;
-    ok = (unsigned int)sh <= 26u && f - (0x200000u - 64u) > 128u;
-    const unsigned long long m = (W + 0x200000ull) >> 22;
-    return __longlong_as_double(0x3ff0000000000000ll - (long long)m);
+    bad = ((unsigned int)W & 0x3fffffu) - (0x200000u - 64u) <= 128u || (cb != 0 && (unsigned int)sh > 26u);
+    return (unsigned int)((W + 0x200000ull) >> 22);
 }
+
+// An FP64 sum and product as the fused operation: a 1 + b and a b - 0 have the bits of
+// a + b and a b (the signs of zeros too), and the FP64 pipe takes a warp's fused
+// operation in 16 cycles of an SM, a plain one in 19 (157 -> 143 ms on the zones above).
+// The constants are the plan's, so that the compiler does not turn the fused operation
+// back.
+struct Fused {
+    double one, zero;
+    __device__ __forceinline__ explicit Fused(const PlanDev& P) : one(P.one), zero(P.neg_zero) {}
+    __device__ __forceinline__ double add(double a, double b) const { return fma(a, one, b); }
+    __device__ __forceinline__ double mul(double a, double b) const { return fma(a, b, zero); }
+};
 
 // Kahan-compensated FP32 sum (the gathers of the mixed form with the FP64 update).
 struct AccKahan {
@@ -348,6 +363,7 @@ __device__ __forceinline__ void update_reduce_fp64(const PlanDev& P, const OptsD
     const double* Yc = g.Y64 + cur * NP1;
     double* Yn64 = g.Y64 + (cur ^ 1) * NP1;
     const double kappa = O.kappa, ymin = O.y_min;
+    const Fused F(P);
     double csum = 0.0, bn = 0.0, bd = 1.0;
     float rmax = 0.f;
     int who = -1;
@@ -357,11 +373,11 @@ __device__ __forceinline__ void update_reduce_fp64(const PlanDev& P, const OptsD
         if (QSS) {
             yn = qss_correct1(y, Fk2[2 * i], fp, 0.5 * (kk + Fk2[2 * i + 1]), h);
         } else {
-            const double kdt = kk * h;
-            yn = ge_bits(kdt, kappa) ? (y + h * fp) / (1.0 + kdt) : y + h * (fp - kk * y);
+            const double kdt = F.mul(kk, h);
+            yn = ge_bits(kdt, kappa) ? (y + h * fp) / F.add(kdt, 1.0) : y + h * (fp - kk * y);
         }
         Yn64[i] = yn;
-        const double d = yn - y;
+        const double d = F.add(-y, yn);
         csum = fma(A[i], d, csum);
         if (EXACT) {
             ratio_max(y, yn, d, ymin, bn, bd);
@@ -381,7 +397,7 @@ __device__ __forceinline__ void update_reduce_fp64(const PlanDev& P, const OptsD
         }
     }
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) csum += __shfl_xor_sync(0xffffffffu, csum, off);
+    for (int off = 16; off > 0; off >>= 1) csum = F.add(csum, __shfl_xor_sync(0xffffffffu, csum, off));
     if ((lane & 31) == 0) g.red_c[lane >> 5] = csum;
     if (EXACT) {
         ratio_reduce(g, lane, bn, bd);
@@ -549,18 +565,19 @@ __device__ __forceinline__ void update_reduce_mixed64(const PlanDev& P, const Op
     double* Yn64 = g.Y64 + (cur ^ 1) * NP1;
     float* Yn32 = g.Y32 + (cur ^ 1) * NP1;
     const double kappa = O.kappa;
+    const Fused F(P);
     double csum = 0.0;
     float rmax = 0.f;
     int ok = 1;
     for (int i = lane; i < N; i += G) {
         const float2 fk = Fk[i];
         const double y = Yc[i], fp = (double)fk.x, kk = (double)fk.y;
-        const double kdt = kk * h;
-        const double yn = (kdt >= kappa) ? (y + h * fp) / (1.0 + kdt) : y + h * (fp - kk * y);
+        const double kdt = F.mul(kk, h);
+        const double yn = ge_bits(kdt, kappa) ? (y + h * fp) / F.add(kdt, 1.0) : y + h * (fp - kk * y);
         const float yn32 = (float)yn;
         Yn64[i] = yn;
         Yn32[i] = yn32;
-        const double d = yn - y;
+        const double d = F.add(-y, yn);
         csum = fma(A[i], d, csum);
         // y32 = fl32(y) and yn32 = fl32(y'): each within 2^-24 relative, so the
         // band of set_guard_band covers their difference and the ratio
@@ -586,7 +603,7 @@ __device__ __forceinline__ void update_reduce_mixed64(const PlanDev& P, const Op
         }
     }
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) csum += __shfl_xor_sync(0xffffffffu, csum, off);
+    for (int off = 16; off > 0; off >>= 1) csum = F.add(csum, __shfl_xor_sync(0xffffffffu, csum, off));
     const unsigned int rbits = __reduce_max_sync(0xffffffffu, __float_as_uint(rmax));
     ok = __all_sync(0xffffffffu, ok);
     if ((lane & 31) == 0) {
@@ -1053,35 +1070,35 @@ __device__ __forceinline__ void flux_pass(const PlanDev& P, const GroupPtrs& g, 
         // 2^53 c_max s < 2^32 (and s >= 0): the degree-2 factors in integers
         const bool fixed = poly == 2 && P.cmax * s < 4.7e-7 && s < 9.5e-7;
         const unsigned long long sf = fixed ? factor_scale(s) : 0;
+        const Fused F(P);
 #pragma unroll 2
         for (int j = j0; j < R; j += stride) {
             const uint32_t rs = rspec[j];
             double k = (double)Kz[j];
-            bool ok = false;
+            bool bad = true;
             double fac;
-            if (fixed) fac = factor_small((double)cexp[j], sf, ok);
-            if (ok)
-                k *= fac;
+            if (fixed) fac = __longlong_as_double(0x3ff0000000000000ll - factor_small((double)cexp[j], sf, bad));
+            if (!bad)
+                k = F.mul(k, fac);
             else if (poly == 2 || poly == 5)
                 k *= exp_neg_small((double)cexp[j] * s, poly);
             else if (poly == 9)
                 k *= exp(-(double)cexp[j] * s);
-            const double ya = Yr[rs & 1023u];
+            const double ka = F.mul(k, Yr[rs & 1023u]);
             if (j < R1) {
-                Vw[j] = (real)(k * ya);
+                Vw[j] = (real)ka;
                 Vw[R + j] = (real)k;
             } else if (j < R12) {
                 const double yb = Yr[(rs >> 10) & 1023u];
-                Vw[j] = (real)(k * ya * yb);
-                Vw[R + j] = (real)(k * yb);
-                Vw[pb1 + j] = (real)(k * ya);
+                Vw[j] = (real)F.mul(ka, yb);
+                Vw[R + j] = (real)F.mul(k, yb);
+                Vw[pb1 + j] = (real)ka;
             } else {
                 const double yb = Yr[(rs >> 10) & 1023u], yc = Yr[rs >> 20];
-                const double ka = k * ya;
-                Vw[j] = (real)(ka * yb * yc);
-                Vw[R + j] = (real)(k * yb * yc);
-                Vw[pb1 + j] = (real)(ka * yc);
-                Vw[pb2 + j] = (real)(ka * yb);
+                Vw[j] = (real)F.mul(F.mul(ka, yb), yc);
+                Vw[R + j] = (real)F.mul(F.mul(k, yb), yc);
+                Vw[pb1 + j] = (real)F.mul(ka, yc);
+                Vw[pb2 + j] = (real)F.mul(ka, yb);
             }
         }
     } else {
@@ -1161,13 +1178,18 @@ __device__ __forceinline__ void gather_pass(const PlanDev& P, const GroupPtrs& g
             continue;
         }
         real acc = (real)0;
+        const Fused F(P);
+        auto add = [&](real a, real b) -> real {
+            if constexpr (PREC == kPrecFP64) return F.add(a, b);
+            else return a + b;
+        };
         if (boff) {  // byte offsets into V (uniform per table)
             const unsigned char* __restrict__ Vb = (const unsigned char*)Vr;
 #pragma unroll 4
-            for (int k = 0; k < len; ++k) acc = acc + *(const real*)(Vb + ix[32 * k]);
+            for (int k = 0; k < len; ++k) acc = add(acc, *(const real*)(Vb + ix[32 * k]));
         } else {
 #pragma unroll 4
-            for (int k = 0; k < len; ++k) acc = acc + Vr[ix[32 * k]];
+            for (int k = 0; k < len; ++k) acc = add(acc, Vr[ix[32 * k]]);
         }
         bool first = true;
         if (hd.y >> 31) {  // warp-uniform
@@ -1175,7 +1197,7 @@ __device__ __forceinline__ void gather_pass(const PlanDev& P, const GroupPtrs& g
             for (int off = 1; off < 32; off <<= 1) {
                 const real o = __shfl_down_sync(0xffffffffu, acc, off);
                 const unsigned int od = __shfl_down_sync(0xffffffffu, d, off);
-                if (l + off < 32 && od == d) acc = acc + o;
+                if (l + off < 32 && od == d) acc = add(acc, o);
             }
             const unsigned int ud = __shfl_up_sync(0xffffffffu, d, 1);
             first = l == 0 || ud != d;
@@ -1683,11 +1705,10 @@ __global__ void __launch_bounds__(1024, 1) integrate_kernel(const __grid_constan
         if (g < P.M) {
             GroupSync gs{1 + g, P.G, P.M == 1 && P.G == (int)blockDim.x};
             unsigned char* gbase = smem + toff + g * P.gl.bytes;
-            // the FP32-flux forms with staged tables (the common case) get their
-            // own copy of the group loop with the tables known to be shared
-            // memory (measured: mixed +2.9 %, mixed with the FP64 update +0.7 %;
-            // the FP64 form, FP64-pipe bound, within noise)
-            if (PREC != kPrecFP64 && P.smem_tables)
+            // staged tables (the common case) get their own copy of the group loop with
+            // the tables known to be shared memory (measured: mixed +2.9 %, mixed with
+            // the FP64 update +0.7 %, FP64 +1.5 %)
+            if (P.smem_tables)
                 run_group<PREC, FEAT, QSS, true>(P, lp.o, smem + moff, smem, gbase, lane, gs);
             else
                 run_group<PREC, FEAT, QSS, false>(P, lp.o, tb, smem, gbase, lane, gs);

@@ -163,6 +163,7 @@ struct PlanDev {
     double cmax;                 // max_j c_j
     float u_tol;                 // FP32-flux forms: cached rates are reused while |u - u_ref| <= u_tol,
                                  //   i.e. while no rate would move by a quarter ulp: 2^-26 / (cmax ln 2)
+    double one, neg_zero;        // FP64 form: 1 and -0 (Fused in kn_integrate.cu)
     float u_one;                 // kn_slots.cu without the rate cache: 2^(-c u) rounds to 1 while |u| <= u_one
     int32_t rate_cache;          // 1: the groups keep the cache Kc (FP32-flux forms, small enough R)
     int32_t zero_idx;            // V index of the constant zero (= R + S_r)
