@@ -688,6 +688,7 @@ static kn_status prepare_launch(kn_network* const* nets, int n_nets, const kn_op
         P.u_one = one_tol(n->cmax);
         P.one = 1.0;
         P.neg_zero = -0.0;
+        P.wide = 0;
         P.rate_cache = rate_cache_on(n, prec) ? 1 : 0;
         P.N = n->N;
         P.R = n->R;
@@ -720,6 +721,32 @@ static kn_status prepare_launch(kn_network* const* nets, int n_nets, const kn_op
         max_smem = std::max(max_smem, t.bytes);
         work[p] = (double)n->Z * (n->R + n->S_r + n->S_p) / (double)t.M;
         total_work += work[p];
+    }
+    // The forms with FP64 in the step, a tiling chosen above for one network without
+    // features (records, the learned proposal): no more groups a CTA than its share of the
+    // zones, so that few zones spread over the SMs (150 zones of 150/1604, FP64 form: 63 ->
+    // 26 ms); and up to two zones an SM the FP64 form's groups are wide, where no lane holds
+    // two species (the sums keep the order of t.G threads): 26.5 -> 25.0 ms, 300 zones 27.1
+    // -> 25.7, one zone 12.7 -> 10.9.  Three fill the FP64 units as they are (60.4 against 60.9).
+    if (prec != kPrecMixed && n_nets == 1 && !o->threads_per_cta && !o->threads_per_zone && !probe && !learn &&
+        !record) {
+        PlanDev& P = lp.plans[0];
+        const int need = std::max(1, (P.n_zones + di.sms - 1) / di.sms);
+        if (need < P.M) {
+            P.M = need;
+            P_best = P.M * P.G;
+            max_smem = (P.smem_tables ? P.tl.bytes : 0) + P.M * P.gl.bytes;
+        }
+        const int W = prec == kPrecFP64 && need <= 2 ? wide_group(P.G) : 0;
+        const GroupLayout gl = group_layout(nets[0], prec, W, extras);
+        const int bytes = (P.smem_tables ? P.tl.bytes : 0) + P.M * gl.bytes;
+        if (W > P.G && P.G >= 64 && P.N <= P.G && P.M * W <= 1024 && P.M * P.G == P_best && bytes <= budget) {
+            P.G = W;
+            P.wide = 1;
+            P.gl = gl;
+            P_best = P.M * W;
+            max_smem = std::max(max_smem, bytes);
+        }
     }
     const int max_block = P_best;
     // one block size for the launch: every plan must fill it exactly

@@ -1137,10 +1137,12 @@ __device__ __forceinline__ void gather_pass(const PlanDev& P, const GroupPtrs& g
     const real* V = (const real*)g.V;
     const int w = lane >> 5, l = lane & 31;
     const int s1 = g.wsl[w + 1];
+    const uint16_t* __restrict__ deal = g.wsl + (P.G >> 5) + 1;  // FP64 form, wide groups
     const bool boff = P.tl.sidx_bytes != 0;
     unsigned char* __restrict__ Fb = Fb_;
     const real* __restrict__ Vr = V;
-    for (int sl = g.wsl[w]; sl < s1; ++sl) {
+    for (int q = g.wsl[w]; q < s1; ++q) {
+        const int sl = PREC == kPrecFP64 && P.wide ? deal[q] : q;
         const uint2 hd = g.shdr[sl];
         const uint16_t* __restrict__ ix = g.sidx + hd.x + l;
         const int len = (int)(hd.y & 0x7fffffffu);
@@ -1221,7 +1223,7 @@ __device__ __forceinline__ void run_group(const PlanDev& P, const OptsDev& O, co
     g.A = tb + P.tl.off_A;
     g.rspec = (const uint32_t*)(tb + P.tl.off_rspec);
     g.cexp = tb + P.tl.off_cexp;
-    g.wsl = (const uint16_t*)(tb + P.tl.off_wsl);
+    g.wsl = (const uint16_t*)(tb + (PREC == kPrecFP64 && P.wide ? P.tl.off_deal : P.tl.off_wsl));
     g.shdr = (const uint2*)(tb + P.tl.off_shdr);
     g.sdst = (const uint16_t*)(tb + P.tl.off_sdst);
     g.sidx = (const uint16_t*)(tb + P.tl.off_sidx);
@@ -1701,7 +1703,10 @@ __global__ void __launch_bounds__(1024, 1) integrate_kernel(const __grid_constan
             toff += P.tl.bytes;
         }
         __syncthreads();
-        const int g = threadIdx.x / P.G, lane = threadIdx.x - g * P.G;
+        const int g = threadIdx.x / P.G;
+        int lane = threadIdx.x - g * P.G;
+        // wide groups: the species warps begin on another scheduler in each group
+        if (PREC == kPrecFP64 && P.wide) lane = lane >= 32 * g ? lane - 32 * g : lane - 32 * g + P.G;
         if (g < P.M) {
             GroupSync gs{1 + g, P.G, P.M == 1 && P.G == (int)blockDim.x};
             unsigned char* gbase = smem + toff + g * P.gl.bytes;

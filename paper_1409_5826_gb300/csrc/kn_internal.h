@@ -56,7 +56,17 @@ struct TableLayout {
     int32_t off_sidx;     // uint16[sum_s 32 len_s]: terms, lane-interleaved: byte offsets into V
                           //   when sidx_bytes, else V indices
     int32_t sidx_bytes;   // 1: sidx holds byte offsets
+    int32_t n_slices;
+    int32_t off_deal;     // FP64 form: the slices dealt to wide_group(G) / 32 warps: uint16 ranges
+                          //   [warps + 1] into the slice numbers [n_slices] that follow
 };
+
+// FP64 form: the threads of a group whose tables are for G threads.  Each of an SM's
+// four schedulers has its own FP64 unit (a warp's instruction takes 64 cycles of it),
+// and warp w runs on scheduler w mod 4, so a group of 5 warps leaves two units idle
+// half of the time: the next multiple of four warps shares the flux pass and the
+// gather's slices evenly.  The sums keep the order of G threads.
+constexpr int wide_group(int G) { return (G + 127) / 128 * 128; }
 
 // Per-group shared-memory layout (byte offsets inside one group's region).
 struct GroupLayout {
@@ -163,6 +173,7 @@ struct PlanDev {
     double cmax;                 // max_j c_j
     float u_tol;                 // FP32-flux forms: cached rates are reused while |u - u_ref| <= u_tol,
                                  //   i.e. while no rate would move by a quarter ulp: 2^-26 / (cmax ln 2)
+    int wide;                    // FP64 form: G is wide_group of the tables' thread count
     double one, neg_zero;        // FP64 form: 1 and -0 (Fused in kn_integrate.cu)
     float u_one;                 // kn_slots.cu without the rate cache: 2^(-c u) rounds to 1 while |u| <= u_one
     int32_t rate_cache;          // 1: the groups keep the cache Kc (FP32-flux forms, small enough R)

@@ -325,6 +325,31 @@ kn_status build_tables_host(const kn_network* n, int prec, int Q, std::vector<un
     off = pad16(off + 2 * (int)sdst.size());
     tl.off_sidx = off;
     off = pad16(off + 2 * (int)sidx.size());
+    // the slices dealt to a wide group's warps, longest first: to the scheduler (w mod 4)
+    // with the least to do, and there to the warp with the least
+    std::vector<uint16_t> deal;
+    tl.n_slices = n_slices;
+    tl.off_deal = off;
+    if (prec == kPrecFP64) {
+        const int D = wide_group(G) / 32;
+        std::vector<int> by(n_slices), load(D, 0), sched(4, 0);
+        auto cost_of = [&](int s) { return (int)(shdr[2 * s + 1] & 0x7fffffffu) + (shdr[2 * s + 1] >> 31 ? 6 : 0); };
+        for (int s = 0; s < n_slices; ++s) by[s] = s;
+        std::stable_sort(by.begin(), by.end(), [&](int x, int y) { return cost_of(x) > cost_of(y); });
+        std::vector<std::vector<uint16_t>> mine(D);
+        for (int s : by) {
+            int w = (int)(std::min_element(sched.begin(), sched.end()) - sched.begin());
+            for (int v = w; v < D; v += 4)
+                if (load[v] < load[w]) w = v;
+            mine[w].push_back((uint16_t)s);
+            load[w] += cost_of(s);
+            sched[w % 4] += cost_of(s);
+        }
+        deal.push_back(0);
+        for (int w = 0; w < D; ++w) deal.push_back((uint16_t)(deal.back() + mine[w].size()));
+        for (auto& m : mine) deal.insert(deal.end(), m.begin(), m.end());
+        off = pad16(off + 2 * (int)deal.size());
+    }
     tl.bytes = off;
     blob.assign(off, 0);
     for (int i = 0; i < N; ++i) {
@@ -354,6 +379,7 @@ kn_status build_tables_host(const kn_network* n, int prec, int Q, std::vector<un
     memcpy(blob.data() + tl.off_shdr, shdr.data(), 4 * shdr.size());
     memcpy(blob.data() + tl.off_sdst, sdst.data(), 2 * sdst.size());
     memcpy(blob.data() + tl.off_sidx, sidx.data(), 2 * sidx.size());
+    if (!deal.empty()) memcpy(blob.data() + tl.off_deal, deal.data(), 2 * deal.size());
     tl.sidx_bytes = byte_off ? 1 : 0;
     T.tl = tl;
     T.L = L_best;

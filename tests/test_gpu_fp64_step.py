@@ -95,3 +95,22 @@ def test_accept_test_bits(kn, name, method):
         g.close()
     for k in ("Y", "t", "dt_next", "steps", "rejects", "status"):
         assert np.array_equal(r[0][k], r[1][k]), k
+
+
+@pytest.mark.parametrize("zones", [1, 5, 153, 311])
+@pytest.mark.parametrize("prec", [0, 2])
+@pytest.mark.parametrize("species,G", [(40, 128), (130, 160), (150, 160), (300, 320)])
+def test_few_zones_keep_their_bits(kn, species, G, prec, zones):
+    # the chosen tiling spreads few zones over the SMs and widens the FP64 form's groups;
+    # an explicit one of the same summation order does neither
+    net = net150() if species == 150 else sweep_network(species)
+    z = profile_zones(net, zones, base_seed=6, t_end=3e-12)
+    out = []
+    for tiling in ({}, {"threads_per_zone": G, "threads_per_cta": G}):
+        g = kn.Network(net)
+        g.set_zones(z)
+        kn.integrate_batch([g], kn.Opts(precision=prec, max_steps=400, **tiling))
+        out.append(g.get())
+        g.close()
+    for k in ("Y", "t", "dt_next", "steps", "rejects", "status"):
+        assert np.array_equal(out[0][k], out[1][k]), k
