@@ -1185,54 +1185,75 @@ __device__ __forceinline__ void run_plan(const PlanDev& P, const OptsDev& O, con
     }
 }
 
-// CK: the capacities of the one plan, or kCapMany: any mix of plans
+// One of several plans.  Its index is a constant, so that the plan's fields are operands
+// in constant memory; through an index they were loads and spilled registers (150/1604
+// alone, 1024 zones to 1e-9 s: 600 ms against 467; 365/4400, 512 zones: 522 against 304).
+template <int NZ, bool QSS, int I>
+__device__ __forceinline__ void run_cap(const LaunchParams& lp, const SlotBase g, SlotCtl& C, int gr, int tid) {
+    const PlanDev& P = lp.plans[I];
+    if (P.cap == kCapWarp) run_plan<NZ, QSS, kCapWarp>(P, lp.o, g, C, gr, tid);
+    else if (P.cap == kCapWide) run_plan<NZ, QSS, kCapWide>(P, lp.o, g, C, gr, tid);
+    else run_plan<NZ, QSS, kCapGroup>(P, lp.o, g, C, gr, tid);
+}
+static_assert(kMaxPlans == 4, "the kernel's constant plan indices");
+
+// CK: the capacities of the one plan, or kCapMany: any mix of plans.  A CTA works on one
+// plan: its home plan or, for the CTAs past the first that every SM gets (one fits on an
+// SM, so these start where another has ended), one that still has zones in its queue.
+// (A loop over the plans in one CTA let the compiler move every plan's set-up out of the
+// loop and keep it there in registers and local memory.)  16, 150 and 365 species, 2048
+// zones: 690 -> 500 ms with both.  Every plan is served: a CTA past the first ones tries
+// the plans from the one of its own number on, and ends only where no queue has a zone.
 template <int NZ, bool QSS, int CK>
 __global__ void __launch_bounds__(kSlotThreads, 1) slots_kernel(const __grid_constant__ LaunchParams lp) {
     extern __shared__ __align__(128) unsigned char smem[];
     __shared__ int s_go;
     constexpr bool ONE = CK != kCapMany;
-    const int np = ONE ? 1 : lp.n_plans;
-    int home = 0;
-    if (!ONE)
-        for (int p = 0; p < np; ++p)
-            if ((int)blockIdx.x >= lp.plans[p].cta_begin && (int)blockIdx.x < lp.plans[p].cta_end) home = p;
-    for (int a = 0; a < np; ++a) {
-        const PlanDev& P = lp.plans[ONE ? 0 : (home + a) % np];
-        if (threadIdx.x == 0)
-            s_go = a == 0 ? (int)blockIdx.x - P.cta_begin < P.n_zones : P.dealt + *((volatile int*)P.queue_head) < P.n_zones;
-        __syncthreads();
-        const int go = s_go;
-        __syncthreads();
-        if (!go) continue;
-        {
-            const int4* src = (const int4*)P.slot_blob;
-            int4* dst = (int4*)smem;
-            for (int i = threadIdx.x; i < P.st.bytes / 16; i += blockDim.x) dst[i] = src[i];
+    if (threadIdx.x == 0) {
+        const int np = ONE ? 1 : lp.n_plans;
+        int home = -1;  // none: no zone is left
+        for (int p = 0; p < np; ++p) {
+            const PlanDev& P = lp.plans[p];
+            const int b = (int)blockIdx.x - P.cta_begin;
+            if (b >= 0 && (int)blockIdx.x < P.cta_end && b < P.n_zones) home = p;
         }
-        __syncthreads();
-        const int gr = threadIdx.x / P.T, tid = threadIdx.x - gr * P.T;
-        if (gr < P.ng) {
-            unsigned char* gb = smem + P.st.bytes + gr * P.sl.bytes;
-            SlotCtl& C = *(SlotCtl*)(gb + P.sl.off_ctl);
-            const SlotBase g{saddr(smem), saddr(gb)};
-            if (tid < NZ) {
-                sts(g.gb + P.sl.off_V + 4 * P.st.zero + 128 * tid, 0.f);
-                sts(g.gb + P.sl.off_Y + at<NZ>(P.N) + 128 * tid, 1.f);  // the factor of an absent reactant
-                C.h[tid] = 0.f;
-                C.u[tid] = 0.f;
-                C.zone[tid] = -2;
-                if (tid == 0) C.live = 0;
-            }
-            // (change_zones begins with a barrier)
-            if constexpr (ONE) {
-                run_plan<NZ, QSS, CK>(P, lp.o, g, C, gr, tid);
-            } else {
-                if (P.cap == kCapWarp) run_plan<NZ, QSS, kCapWarp>(P, lp.o, g, C, gr, tid);
-                else if (P.cap == kCapWide) run_plan<NZ, QSS, kCapWide>(P, lp.o, g, C, gr, tid);
-                else run_plan<NZ, QSS, kCapGroup>(P, lp.o, g, C, gr, tid);
-            }
+        for (int a = 0; a < np && !ONE && home < 0; ++a) {
+            const PlanDev& P = lp.plans[((int)blockIdx.x + a) % np];
+            if (P.dealt + *((volatile int*)P.queue_head) < P.n_zones) home = ((int)blockIdx.x + a) % np;
         }
-        __syncthreads();
+        s_go = home;
+    }
+    __syncthreads();
+    const int i = s_go;
+    if (i < 0) return;
+    const PlanDev& P = lp.plans[ONE ? 0 : i];
+    {
+        const int4* src = (const int4*)P.slot_blob;
+        int4* dst = (int4*)smem;
+        for (int k = threadIdx.x; k < P.st.bytes / 16; k += blockDim.x) dst[k] = src[k];
+    }
+    __syncthreads();
+    const int gr = threadIdx.x / P.T, tid = threadIdx.x - gr * P.T;
+    if (gr >= P.ng) return;
+    unsigned char* gb = smem + P.st.bytes + gr * P.sl.bytes;
+    SlotCtl& C = *(SlotCtl*)(gb + P.sl.off_ctl);
+    const SlotBase g{saddr(smem), saddr(gb)};
+    if (tid < NZ) {
+        sts(g.gb + P.sl.off_V + 4 * P.st.zero + 128 * tid, 0.f);
+        sts(g.gb + P.sl.off_Y + at<NZ>(P.N) + 128 * tid, 1.f);  // the factor of an absent reactant
+        C.h[tid] = 0.f;
+        C.u[tid] = 0.f;
+        C.zone[tid] = -2;
+        if (tid == 0) C.live = 0;
+    }
+    // (change_zones begins with a barrier)
+    if constexpr (ONE) {
+        run_plan<NZ, QSS, CK>(P, lp.o, g, C, gr, tid);
+    } else {
+        if (i == 0) run_cap<NZ, QSS, 0>(lp, g, C, gr, tid);
+        else if (i == 1) run_cap<NZ, QSS, 1>(lp, g, C, gr, tid);
+        else if (i == 2) run_cap<NZ, QSS, 2>(lp, g, C, gr, tid);
+        else run_cap<NZ, QSS, 3>(lp, g, C, gr, tid);
     }
 }
 
@@ -1254,7 +1275,7 @@ SlotsFn slots_fn(int nz, bool qss, int cap) {
 
 cudaError_t launch_slots(const LaunchParams& lp, int grid, int block, cudaStream_t stream) {
     const int cap = lp.n_plans > 1 ? kCapMany : lp.plans[0].cap;
-    slots_fn(lp.nz, lp.o.method != 0, cap)<<<grid, block, lp.smem_bytes, stream>>>(lp);
+    slots_fn(lp.nz, lp.o.method != 0, cap)<<<grid * lp.n_plans, block, lp.smem_bytes, stream>>>(lp);
     return cudaGetLastError();
 }
 

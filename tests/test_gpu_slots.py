@@ -106,3 +106,32 @@ def test_same_bits_small_odd_networks(env):
         z = Zones(Y0=np.tile(net.initial_Y(), (4, 1)), T0=np.ones(4), rho0=np.linspace(1, 2, 4), tau=np.zeros(4),
                   t_start=np.zeros(4), t_end=np.full(4, 0.2), dt_trial=np.full(4, 1e-6))
         _both(env, net, z, 32 if seed % 2 else 64)
+
+
+@pytest.mark.parametrize("zones", [(1, 1, 1), (2, 40, 1), (900, 3, 160), (0, 310, 5), (7, 1, 2, 3), (60, 200, 33, 90)])
+def test_same_bits_with_several_networks(env, zones):
+    # networks of several sizes in one launch, some with fewer zones than CTAs of their own
+    torch, kn = env
+    G = 384
+    nets = [chain_network(), net150(), net365(), sweep_network(64)][:len(zones)]
+    opts = kn.Opts(precision=kn.PREC_MIXED, threads_per_zone=G, threads_per_cta=G, max_steps=20000)
+    gs, dzs = [], []
+    for net, Z in zip(nets, zones):
+        if not Z:
+            continue
+        z = profile_zones(net, Z, base_seed=33, t_end=3e-12)
+        gs.append((net, Z, kn.Network(net)))
+        dzs.append({k: torch.from_numpy(np.ascontiguousarray(getattr(z, k))).cuda() for k in IN})
+        gs[-1][2].set_zones(dzs[-1])
+    kn.integrate_batch([g for _, _, g in gs], opts)
+    for (net, Z, g), dz in zip(gs, dzs):
+        a = g.get()
+        one = kn.Network(net)
+        one.set_zones(dz)
+        kn.integrate_batch([one], opts)
+        b = one.get()
+        for k in OUT:
+            assert np.array_equal(a[k], b[k]), (k, net.n_species)
+        assert (a["status"] == 0).all()
+        g.close()
+        one.close()
