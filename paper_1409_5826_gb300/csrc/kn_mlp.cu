@@ -85,7 +85,7 @@ __device__ __forceinline__ void warp_mma(float (&c)[NT][4], const bf16* A, int l
                                          int n0, int K, int lane) {
     const int r = lane & 7, q = lane >> 3;
     const int lo8 = (q & 1) << 3, hi8 = (q & 2) << 2;  // matrix q: +8 on its first / second index
-#pragma unroll 2
+#pragma unroll 4
     for (int k0 = 0; k0 < K; k0 += 16) {
         uint32_t a[4];
         if (A_ROW)  // matrices (m, k): (0,0) (8,0) (0,8) (8,8)
@@ -114,10 +114,15 @@ constexpr int kTileRows = 64;
 // row stride of the per-tile partial gradients: the parameter count padded to
 // 16 bytes, so every tile's row keeps the float2 stores 8-byte aligned
 constexpr int kPartStride = (kMlpParams + 3) & ~3;
-constexpr int kTileThreads = 256;  // 8 warps
+// 16 warps: a tile's passes are chains of shared-memory loads, matrix instructions and
+// barriers, and twice the warps halve each.  With that, every load of the staging in
+// flight at once, the output rows side by side, dZ2 eight columns at a time and the
+// column sums on all threads, a tile takes 14.2 us instead of 20.8 (64 tiles of 64
+// rows); the matrix instructions' own rate bounds it to 5.
+constexpr int kTileThreads = 512;
 constexpr int LDF = NF + 8, LDN = NH + 8;  // padded row strides (BF16 elements)
 constexpr int kTileSmem = (NF * LDN + NH * LDN + kTileRows * LDF + 4 * kTileRows * LDN) * 2 +
-                          (3 * NH + 2 * kTileRows + 8 + 2 * kTileThreads / 32) * 4;
+                          (3 * NH + 3 * kTileRows) * 4;
 
 template <bool BWD>
 __global__ void __launch_bounds__(kTileThreads, 1)
@@ -137,49 +142,63 @@ mlp_tile(const float* __restrict__ feat, const float* __restrict__ y, int B, con
     float* w3s = b2s + NH;
     float* outs = w3s + NH;                // [rows]
     float* douts = outs + kTileRows;       // [rows]
-    float* red = douts + kTileRows;        // [8] + per-warp sums
+    float* errs = douts + kTileRows;       // [rows]
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int r0 = blockIdx.x * kTileRows;
     const int rows = min(kTileRows, B - r0);
 
     // stage the BF16 weights, the FP32 biases and the normalised inputs
-    for (int i = tid; i < NF * (NH / 8); i += kTileThreads) {
-        const int k = i / (NH / 8), c = i - k * (NH / 8);
-        *(int4*)(W1s + k * LDN + 8 * c) = *(const int4*)(Wb + k * NH + 8 * c);
-    }
-    for (int i = tid; i < NH * (NH / 8); i += kTileThreads) {
-        const int k = i / (NH / 8), c = i - k * (NH / 8);
-        *(int4*)(W2s + k * LDN + 8 * c) = *(const int4*)(Wb + NF * NH + k * NH + 8 * c);
-    }
-    for (int i = tid; i < NH; i += kTileThreads) {
-        b1s[i] = P[OFF_B1 + i];
-        b2s[i] = P[OFF_B2 + i];
-        w3s[i] = P[OFF_W3 + i];
-    }
-    for (int i = tid; i < kTileRows * (NF / 4); i += kTileThreads) {
-        const int m = i / (NF / 4), c = i - m * (NF / 4);
-        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (m < rows) {
-            v = *(const float4*)(feat + (size_t)(r0 + m) * NF + 4 * c);
-            v.x = (v.x - norm[4 * c]) * norm[NF + 4 * c];
-            v.y = (v.y - norm[4 * c + 1]) * norm[NF + 4 * c + 1];
-            v.z = (v.z - norm[4 * c + 2]) * norm[NF + 4 * c + 2];
-            v.w = (v.w - norm[4 * c + 3]) * norm[NF + 4 * c + 3];
+    {
+        constexpr int C = NH / 8, NW = (NF + NH) * C / kTileThreads, NX = kTileRows * (NF / 4) / kTileThreads;
+        static_assert((NF + NH) * C % kTileThreads == 0 && kTileRows * (NF / 4) % kTileThreads == 0, "staging");
+        int4 wv[NW];
+        float4 xv[NX];
+        // every load of the thread before the first store: one round trip instead of one a loop
+        // (Wb holds W1's rows, then W2's)
+#pragma unroll
+        for (int q = 0; q < NW; ++q) wv[q] = ((const int4*)Wb)[tid + q * kTileThreads];
+#pragma unroll
+        for (int q = 0; q < NX; ++q) {
+            const int i = tid + q * kTileThreads, m = i / (NF / 4), c = i % (NF / 4);
+            xv[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (m < rows) {
+                float4 v = *(const float4*)(feat + (size_t)(r0 + m) * NF + 4 * c);
+                const float4 mu = *(const float4*)(norm + 4 * c), is = *(const float4*)(norm + NF + 4 * c);
+                v.x = (v.x - mu.x) * is.x;
+                v.y = (v.y - mu.y) * is.y;
+                v.z = (v.z - mu.z) * is.z;
+                v.w = (v.w - mu.w) * is.w;
+                xv[q] = v;
+            }
         }
-        __nv_bfloat162* d = (__nv_bfloat162*)(Xs + m * LDF + 4 * c);
-        d[0] = __floats2bfloat162_rn(v.x, v.y);
-        d[1] = __floats2bfloat162_rn(v.z, v.w);
+        if (tid < NH) {
+            b1s[tid] = P[OFF_B1 + tid];
+            b2s[tid] = P[OFF_B2 + tid];
+            w3s[tid] = P[OFF_W3 + tid];
+        }
+#pragma unroll
+        for (int q = 0; q < NW; ++q) {  // W2s follows W1s, with the same row stride
+            const int i = tid + q * kTileThreads;
+            *(int4*)(W1s + (i / C) * LDN + 8 * (i % C)) = wv[q];
+        }
+#pragma unroll
+        for (int q = 0; q < NX; ++q) {
+            const int i = tid + q * kTileThreads;
+            __nv_bfloat162* d = (__nv_bfloat162*)(Xs + (i / (NF / 4)) * LDF + 4 * (i % (NF / 4)));
+            d[0] = __floats2bfloat162_rn(xv[q].x, xv[q].y);
+            d[1] = __floats2bfloat162_rn(xv[q].z, xv[q].w);
+        }
     }
     __syncthreads();
 
     const int g = lane >> 2, t = lane & 3;
-    const int wm = (w & 3) * 16, wn = (w >> 2) * 64;  // 64 x 128 outputs: 4 x 2 warp tiles
+    const int wm = (w & 3) * 16, wn = (w >> 2) * 32;  // 64 x 128 outputs: 4 x 4 warp tiles
     // H = ReLU(A W + b), BF16, for the 64 x 128 warp-tiled outputs
     auto dense_relu = [&](const bf16* A, int lda, const bf16* W, int K, const float* bias, bf16* H) {
-        float c[8][4] = {};
-        warp_mma<8, true, true>(c, A, lda, wm, W, LDN, wn, K, lane);
+        float c[4][4] = {};
+        warp_mma<4, true, true>(c, A, lda, wm, W, LDN, wn, K, lane);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int j = 0; j < 4; ++j) {
             const int n = wn + 8 * j + 2 * t;
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
@@ -193,47 +212,77 @@ mlp_tile(const float* __restrict__ feat, const float* __restrict__ y, int B, con
     __syncthreads();
     dense_relu(H1s, LDN, W2s, NH, b2s, H2s);
     __syncthreads();
-    // out = H2 w3 + b3 (FP32), 8 rows per warp
+    // out = H2 w3 + b3 (FP32), the rows of a warp side by side
     const float b3 = P[OFF_B3];
-    float se = 0.f;
-    for (int m = w * (kTileRows / 8); m < (w + 1) * (kTileRows / 8); ++m) {
-        float s = 0.f;
-        for (int n = lane; n < NH; n += 32) s = fmaf(__bfloat162float(H2s[m * LDN + n]), w3s[n], s);
+    {
+        constexpr int RW = kTileRows / (kTileThreads / 32);
+        float s[RW];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        const float o_m = s + b3;
-        if (lane == 0) {
-            if (!BWD) {
-                if (m < rows) out[r0 + m] = o_m;
-            } else {
-                const float e = m < rows ? o_m - y[r0 + m] : 0.f;
-                outs[m] = o_m;
-                douts[m] = 2.f * e / (float)B;
-                se = fmaf(e, e, se);
+        for (int q = 0; q < RW; ++q) {
+            s[q] = 0.f;
+#pragma unroll
+            for (int n = 0; n < NH; n += 32)
+                s[q] = fmaf(__bfloat162float(H2s[(w * RW + q) * LDN + n + lane]), w3s[n + lane], s[q]);
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+            for (int q = 0; q < RW; ++q) s[q] += __shfl_xor_sync(0xffffffffu, s[q], o);
+#pragma unroll
+        for (int q = 0; q < RW; ++q) {
+            const int m = w * RW + q;
+            const float o_m = s[q] + b3;
+            if (lane == q) {
+                if (!BWD) {
+                    if (m < rows) out[r0 + m] = o_m;
+                } else {
+                    const float e = m < rows ? o_m - y[r0 + m] : 0.f;
+                    errs[m] = e;
+                    douts[m] = 2.f * e / (float)B;
+                }
             }
         }
     }
     if (!BWD) return;
-    if (lane == 0) red[w] = se;
     __syncthreads();
-    if (tid == 0) {
+    // the tile's squared errors: eight rows a lane, then the lanes in order
+    if (w == 0) {
+        float se = 0.f;
+        if (lane < 8)
+#pragma unroll
+            for (int q = 0; q < 8; ++q) se = fmaf(errs[8 * lane + q], errs[8 * lane + q], se);
         float l = 0.f;
-        for (int i = 0; i < kTileThreads / 32; ++i) l += red[i];
-        loss_part[blockIdx.x] = l;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) l += __shfl_sync(0xffffffffu, se, q);
+        if (lane == 0) loss_part[blockIdx.x] = l;
     }
-    // dZ2 = dout w3 [H2 > 0]  (BF16)
-    for (int i = tid; i < kTileRows * NH; i += kTileThreads) {
-        const int m = i / NH, n = i - m * NH;
-        const float keep = __bfloat162float(H2s[m * LDN + n]) > 0.f ? 1.f : 0.f;
-        dZ2s[m * LDN + n] = __float2bfloat16(douts[m] * w3s[n] * keep);
+    // dZ2 = dout w3 [H2 > 0]  (BF16), eight columns at a time
+#pragma unroll
+    for (int i = tid; i < kTileRows * (NH / 8); i += kTileThreads) {
+        const int m = i / (NH / 8), n = 8 * (i % (NH / 8));
+        const float d = douts[m];
+        union {
+            int4 v;
+            __nv_bfloat162 h[4];
+        } a, z;
+        a.v = *(const int4*)(H2s + m * LDN + n);
+        const float4 wa = *(const float4*)(w3s + n), wb = *(const float4*)(w3s + n + 4);
+        const float wv[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float2 hv = __bfloat1622float2(a.h[q]);
+            z.h[q] = __floats2bfloat162_rn(d * wv[2 * q] * (hv.x > 0.f ? 1.f : 0.f),
+                                           d * wv[2 * q + 1] * (hv.y > 0.f ? 1.f : 0.f));
+        }
+        *(int4*)(dZ2s + m * LDN + n) = z.v;
     }
     __syncthreads();
     // dZ1 = (dZ2 W2^T) [H1 > 0]  (W2 stored [k][n] is W2^T stored [n][k])
     {
-        float c[8][4] = {};
-        warp_mma<8, true, false>(c, dZ2s, LDN, wm, W2s, LDN, wn, NH, lane);
+        float c[4][4] = {};
+        warp_mma<4, true, false>(c, dZ2s, LDN, wm, W2s, LDN, wn, NH, lane);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int j = 0; j < 4; ++j) {
             const int n = wn + 8 * j + 2 * t;
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
@@ -246,48 +295,50 @@ mlp_tile(const float* __restrict__ feat, const float* __restrict__ y, int B, con
     }
     __syncthreads();
     float* G = part + (size_t)blockIdx.x * kPartStride;
-    // dW1 = X^T dZ1 (64 x 128, K = tile rows): 4 x 2 warp tiles
+    // dW1 = X^T dZ1 (64 x 128, K = tile rows): 4 x 4 warp tiles
     {
-        float c[8][4] = {};
-        warp_mma<8, false, true>(c, Xs, LDF, wm, dZ1s, LDN, wn, kTileRows, lane);
+        float c[4][4] = {};
+        warp_mma<4, false, true>(c, Xs, LDF, wm, dZ1s, LDN, wn, kTileRows, lane);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int j = 0; j < 4; ++j) {
             const int n = wn + 8 * j + 2 * t;
 #pragma unroll
             for (int h = 0; h < 2; ++h)
                 *(float2*)(G + OFF_W1 + (wm + g + 8 * h) * NH + n) = make_float2(c[j][2 * h], c[j][2 * h + 1]);
         }
     }
-    // dW2 = H1^T dZ2 (128 x 128, K = tile rows): warp w takes rows 16 w
+    // dW2 = H1^T dZ2 (128 x 128, K = tile rows): 8 x 2 warp tiles
     {
-        float c[16][4] = {};
-        warp_mma<16, false, true>(c, H1s, LDN, 16 * w, dZ2s, LDN, 0, kTileRows, lane);
+        const int m0 = 16 * (w & 7), n0 = 64 * (w >> 3);
+        float c[8][4] = {};
+        warp_mma<8, false, true>(c, H1s, LDN, m0, dZ2s, LDN, n0, kTileRows, lane);
 #pragma unroll
-        for (int j = 0; j < 16; ++j) {
-            const int n = 8 * j + 2 * t;
+        for (int j = 0; j < 8; ++j) {
+            const int n = n0 + 8 * j + 2 * t;
 #pragma unroll
             for (int h = 0; h < 2; ++h)
-                *(float2*)(G + OFF_W2 + (16 * w + g + 8 * h) * NH + n) = make_float2(c[j][2 * h], c[j][2 * h + 1]);
+                *(float2*)(G + OFF_W2 + (m0 + g + 8 * h) * NH + n) = make_float2(c[j][2 * h], c[j][2 * h + 1]);
         }
     }
     // column sums: b1 = sum dZ1, b2 = sum dZ2, w3 = sum H2 dout, b3 = sum dout
-    if (tid < NH) {
-        float s1 = 0.f, s3 = 0.f;
-        for (int m = 0; m < rows; ++m) {
-            s1 += __bfloat162float(dZ1s[m * LDN + tid]);
-            s3 = fmaf(__bfloat162float(H2s[m * LDN + tid]), douts[m], s3);
+    {
+        const int q = tid / NH, n = tid % NH;
+        const bf16* src = (q == 0 ? dZ1s : (q == 1 ? dZ2s : H2s)) + n;
+        float s = 0.f;
+        auto add = [&](int m) {
+            if (q == 3) s += douts[m];
+            else if (q == 2) s = fmaf(__bfloat162float(src[m * LDN]), douts[m], s);
+            else s += __bfloat162float(src[m * LDN]);
+        };
+        if (q < 3 || n == 0) {
+            if (rows == kTileRows) {
+#pragma unroll 16
+                for (int m = 0; m < kTileRows; ++m) add(m);
+            } else {
+                for (int m = 0; m < rows; ++m) add(m);
+            }
+            G[(q == 0 ? OFF_B1 : (q == 1 ? OFF_B2 : (q == 2 ? OFF_W3 : OFF_B3))) + n] = s;
         }
-        G[OFF_B1 + tid] = s1;
-        G[OFF_W3 + tid] = s3;
-    } else {
-        const int n = tid - NH;
-        float s2 = 0.f, s4 = 0.f;
-        for (int m = 0; m < rows; ++m) {
-            s2 += __bfloat162float(dZ2s[m * LDN + n]);
-            s4 += douts[m];
-        }
-        G[OFF_B2 + n] = s2;
-        if (n == 0) G[OFF_B3] = s4;
     }
 }
 
@@ -297,11 +348,13 @@ __global__ void reduce_partials(const float* __restrict__ part, int T, float* __
     const int p = blockIdx.x * blockDim.x + threadIdx.x;
     if (p < kMlpParams) {
         float s = 0.f;
+#pragma unroll 16
         for (int i = 0; i < T; ++i) s += part[(size_t)i * kPartStride + p];
         G[p] = s;
     }
     if (loss && p == 0) {
         float l = 0.f;
+#pragma unroll 16
         for (int i = 0; i < T; ++i) l += loss_part[i];
         *loss = l * inv_B;
     }
