@@ -784,7 +784,7 @@ static kn_status prepare_launch(kn_network* const* nets, int n_nets, const kn_op
         cnt = std::max(0, std::min(cnt, grid - b));
         lp.plans[p].cta_begin = b;
         lp.plans[p].cta_end = b + cnt;
-        lp.plans[p].dealt = cnt * lp.plans[p].ng * lp.nz;
+        lp.plans[p].dealt = cnt * (slots ? lp.plans[p].ng * lp.nz : lp.plans[p].M);
         b += cnt;
     }
     OptsDev& D = lp.o;
@@ -1045,6 +1045,7 @@ kn_status noalloc_prepare(kn_network* n, const kn_opts* o, int32_t n_zones, cons
     block = P;
     Pd.cta_begin = 0;
     Pd.cta_end = grid;
+    Pd.dealt = grid * Pd.M;
     OptsDev& D = lp.o;
     D.kappa = o->kappa;
     D.eps_r = o->eps_r;

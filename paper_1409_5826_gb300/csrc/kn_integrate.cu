@@ -1213,7 +1213,7 @@ __device__ __forceinline__ void gather_pass(const PlanDev& P, const GroupPtrs& g
 // rather than through generic pointers; the code is the same otherwise.
 template <int PREC, bool FEAT, bool QSS, bool TB_SHARED>
 __device__ __forceinline__ void run_group(const PlanDev& P, const OptsDev& O, const unsigned char* tb, const unsigned char* mlp_smem,
-                          unsigned char* gbase, const int lane, const GroupSync gs) {
+                          unsigned char* gbase, const int gr, const int lane, const GroupSync gs) {
     using real = typename PrecTraits<PREC>::real;
     const int N = P.N, R = P.R, G = P.G, NP1 = N + 1;
     const int R1 = P.R1, R12 = P.R12;
@@ -1257,9 +1257,16 @@ __device__ __forceinline__ void run_group(const PlanDev& P, const OptsDev& O, co
 
     if (lane == 0) V[P.zero_idx] = (real)0;
 
+    // A home CTA's groups start with zones dealt over the CTAs, then over the groups: the
+    // queue's first zones take the most steps, and where the groups of one CTA took them
+    // from the queue side by side, that SM finished last (1024 zones of 150/1604 to
+    // 1e-10 s, FP64 update: 192 -> 140 ms; 512 learned zones: 32.8 -> 30.2).
+    if (lane == 0)
+        S.zone = (int)blockIdx.x >= P.cta_begin && (int)blockIdx.x < P.cta_end ? -2 : -1;
     for (;;) {
         if (lane == 0) {
-            const int q = atomicAdd(P.queue_head, 1);
+            const int q = S.zone == -2 ? gr * (P.cta_end - P.cta_begin) + (int)blockIdx.x - P.cta_begin
+                                       : P.dealt + atomicAdd(P.queue_head, 1);
             S.zone = q < P.n_zones ? P.order[q] : -1;
             S.valid = 1;
             if (O.zone_ns) S.t_fetch_ns = global_ns();
@@ -1688,7 +1695,9 @@ __global__ void __launch_bounds__(1024, 1) integrate_kernel(const __grid_constan
         if ((int)blockIdx.x >= lp.plans[p].cta_begin && (int)blockIdx.x < lp.plans[p].cta_end) home = p;
     for (int a = 0; a < np; ++a) {
         const PlanDev& P = lp.plans[(home + a) % np];
-        if (threadIdx.x == 0) s_go = *((volatile int*)P.queue_head) < P.n_zones;
+        if (threadIdx.x == 0)
+            s_go = a == 0 ? (int)blockIdx.x - P.cta_begin < P.n_zones
+                          : P.dealt + *((volatile int*)P.queue_head) < P.n_zones;
         __syncthreads();
         const int go = s_go;
         __syncthreads();
@@ -1714,9 +1723,9 @@ __global__ void __launch_bounds__(1024, 1) integrate_kernel(const __grid_constan
             // the tables known to be shared memory (measured: mixed +2.9 %, mixed with
             // the FP64 update +0.7 %, FP64 +1.5 %)
             if (P.smem_tables)
-                run_group<PREC, FEAT, QSS, true>(P, lp.o, smem + moff, smem, gbase, lane, gs);
+                run_group<PREC, FEAT, QSS, true>(P, lp.o, smem + moff, smem, gbase, g, lane, gs);
             else
-                run_group<PREC, FEAT, QSS, false>(P, lp.o, tb, smem, gbase, lane, gs);
+                run_group<PREC, FEAT, QSS, false>(P, lp.o, tb, smem, gbase, g, lane, gs);
         }
         __syncthreads();
     }

@@ -114,3 +114,26 @@ def test_few_zones_keep_their_bits(kn, species, G, prec, zones):
         g.close()
     for k in ("Y", "t", "dt_next", "steps", "rejects", "status"):
         assert np.array_equal(out[0][k], out[1][k]), k
+
+
+@pytest.mark.parametrize("zones", [(1, 1), (2, 700), (310, 3), (0, 160)])
+@pytest.mark.parametrize("prec", [0, 2])
+def test_several_networks_keep_their_bits(kn, prec, zones):
+    # the CTAs' first zones are dealt, the others come from the queues
+    opts = kn.Opts(precision=prec, threads_per_zone=160, threads_per_cta=160, max_steps=300)
+    nets = [n for n, Z in zip((chain_network(), net150()), zones) if Z]
+    zs = [profile_zones(n, Z, base_seed=8, t_end=3e-12) for n, Z in zip(nets, [Z for Z in zones if Z])]
+    gs = [kn.Network(n) for n in nets]
+    for g, z in zip(gs, zs):
+        g.set_zones(z)
+    kn.integrate_batch(gs, opts)
+    for net, g, z in zip(nets, gs, zs):
+        one = kn.Network(net)
+        one.set_zones(z)
+        kn.integrate_batch([one], opts)
+        a, b = g.get(), one.get()
+        for k in ("Y", "t", "dt_next", "steps", "rejects", "status"):
+            assert np.array_equal(a[k], b[k]), k
+        assert (a["steps"] > 0).all()
+        g.close()
+        one.close()
