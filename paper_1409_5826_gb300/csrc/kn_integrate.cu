@@ -1323,7 +1323,7 @@ __device__ __forceinline__ void run_group(const PlanDev& P, const OptsDev& O, co
                 S.u_p = 0.f;
                 S.refresh_p = 0;
                 S.u = 0.f;
-                S.u_ref = -1e30f;  // the first flux pass computes the cached rates
+                S.u_ref = -INFINITY;  // the first flux pass computes the cached rates, however wide u_tol is
                 S.steps = 0;
                 S.rejects = 0;
                 S.props = 0;

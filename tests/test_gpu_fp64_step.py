@@ -6,7 +6,8 @@ from fractions import Fraction
 import numpy as np
 import pytest
 
-from kn_inputs import Zones, chain_network, custom_network, net150, profile_zones, sweep_network
+from kn_inputs import (Zones, chain_network, custom_network, net150, pair_network, profile_zones,
+                       sweep_network)
 
 pytestmark = pytest.mark.gpu
 
@@ -137,3 +138,26 @@ def test_several_networks_keep_their_bits(kn, prec, zones):
         assert (a["steps"] > 0).all()
         g.close()
         one.close()
+
+
+@pytest.mark.parametrize("prec", [1, 2])
+def test_rates_without_temperature_dependence(kn, prec):
+    # every rate exponent 0: the cached rates never go stale, and the first pass still forms
+    # them.  Another network's values are left in shared memory first.
+    z = profile_zones(net150(), 300, base_seed=9, t_end=3e-12)
+    g = kn.Network(net150())
+    g.set_zones(z)
+    kn.integrate_batch([g], kn.Opts(precision=prec, max_steps=50, threads_per_zone=160, threads_per_cta=160))
+    g.close()
+    net = pair_network(2.0, 1.0)
+    f = lambda v: np.full(300, float(v))
+    z = Zones(Y0=np.tile([0.9, 0.1], (300, 1)), T0=f(1), rho0=f(1), tau=f(2), t_start=f(0.1), t_end=f(1), dt_trial=f(1e-3))
+    out = []
+    for p in (0, prec):
+        g = kn.Network(net)
+        g.set_zones(z)
+        kn.integrate_batch([g], kn.Opts(precision=p, max_steps=100000))
+        out.append(g.get())
+        g.close()
+    assert np.array_equal(out[0]["steps"], out[1]["steps"])
+    assert np.allclose(out[0]["Y"], out[1]["Y"], rtol=1e-4, atol=0)  # the forms' bar for equal steps
