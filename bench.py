@@ -396,11 +396,19 @@ def timed_batches(kn, nets, set_zones, opts, steps, warmup, stream, flush, zone_
             "zone_ns": zone_ns.cpu().numpy() if zone_ns is not None else None}
 
 
+def zones_in_flight(zone_ns):
+    """The most zones that were in the kernel's slots at one time (a thread group
+    holds one zone or two)."""
+    start, end = np.sort(zone_ns[:, 0]), np.sort(zone_ns[:, 1])
+    # zones that start at or after another's end may take its slot
+    return int((np.arange(1, len(start) + 1) - np.searchsorted(end, start, side="right")).max())
+
+
 def tail_stats(zone_ns, steps, groups):
     """From the per-zone timer stamps of one batch: the batch span, when the
     work queue drained (the last fetch), the time after that (the tail), the
     spread of zone finish times, the longest zone, and the mean occupancy of
-    the zone groups."""
+    the `groups` zone slots."""
     ns = zone_ns.astype(np.float64)
     t0 = ns[:, 0].min()
     fetch = (ns[:, 0] - t0) / 1e6
@@ -419,7 +427,7 @@ def _mean(x):
     return float(np.mean(x))
 
 
-def smem_roofline(parts, kms, clk, n_sms, qss=False):
+def smem_roofline(parts, kms, clk, n_sms, qss=False, kernel="slots_kernel"):
     """Shared-memory roofline of the FP32-flux forms: the measurement plan's
     bytes per accepted zone-step (algorithmic_smem_bytes, FP32 widths) over
     the kernel time, against 128 B/clk/SM x SMs x the sampled SM clock.
@@ -433,7 +441,7 @@ def smem_roofline(parts, kms, clk, n_sms, qss=False):
                                           if qss else 0.0)
              for n, st, rj in parts)
     return {"bound": "alu", "resource": "shared-memory bandwidth (SM-local)", "unit": "GB/s",
-            "kernel": "integrate_kernel", "achieved": b / (kms / 1e3) / 1e9, "peak": peak,
+            "kernel": kernel, "achieved": b / (kms / 1e3) / 1e9, "peak": peak,
             "frac": b / (kms / 1e3) / 1e9 / peak,
             "peak_source": "derived: 128 B/clk/SM x SMs x sampled SM clock",
             "algorithmic_smem_bytes_per_launch": b,
@@ -499,8 +507,7 @@ def other_forms(kn, g, net, zones, dz, stream, flush, mixed_line, args):
     zns = torch.zeros((zones.n_zones, 2), dtype=torch.int64, device=torch.device("cuda", torch.cuda.current_device()))
 
     def tail_of(tb, tuned):
-        groups = n_sms * (tuned["threads_per_cta"] // tuned["threads_per_zone"]) if tuned else None
-        return tail_stats(tb["zone_ns"], g.get(stream)["steps"], groups)
+        return tail_stats(tb["zone_ns"], g.get(stream)["steps"], zones_in_flight(tb["zone_ns"]) if tuned else None)
 
     out["mixed"] = {"median_rel_err_vs_tight_oracle": err(), "see": "the headline value and roofline"}
     # the split the measurement plan names: FP32 rates, fluxes and Kahan
@@ -515,7 +522,8 @@ def other_forms(kn, g, net, zones, dz, stream, flush, mixed_line, args):
     st = tb["stats"]
     roof = fp64_roofline(update_fp64_flops(net, st["steps"] + st["rejects"]), kms, fp64_peak,
                          "11 FP64 operations per species per attempt (update, conservation sum, test)")
-    roof["smem"] = smem_roofline([(net, st["steps"], st["rejects"])], kms, tb["clocks"], n_sms)
+    roof["smem"] = smem_roofline([(net, st["steps"], st["rejects"])], kms, tb["clocks"], n_sms,
+                                 kernel="integrate_kernel")
     out["mixed_fp64_update"] = _form_line(tb, [g], zones.n_zones, roof,
                                           {"median_rel_err_vs_tight_oracle": err(), "tiling": tuned,
                                            "tail": tail_of(tb, tuned)})
@@ -575,7 +583,8 @@ def other_forms(kn, g, net, zones, dz, stream, flush, mixed_line, args):
                        zns)
     st = tb["stats"]
     kms = _mean(tb["kernel_ms"])
-    roof = smem_roofline([(net, st["steps"], st["rejects"])], kms, tb["clocks"], n_sms)
+    roof = smem_roofline([(net, st["steps"], st["rejects"])], kms, tb["clocks"], n_sms,
+                         kernel="integrate_kernel")
     # the network evaluation on CUDA cores: 2 (64 128 + 128 128 + 128) flops
     # per proposal, one proposal per state reached by an accepted step
     mlp_flops = 2.0 * (64 * 128 + 128 * 128 + 128) * (st["steps"] - zones.n_zones)
@@ -893,7 +902,8 @@ def main():
         # widening of F+ and k); the shared-memory figure rides along
         roof = fp64_roofline(update_fp64_flops(net, st["steps"] + st["rejects"]), kms, kn.measure_fp64_peak(stream),
                              "11 FP64 operations per species per attempt (update, conservation sum, test)")
-        roof["smem"] = smem_roofline([(net, st["steps"], st["rejects"])], kms, clk, n_sms)
+        roof["smem"] = smem_roofline([(net, st["steps"], st["rejects"])], kms, clk, n_sms,
+                                     kernel="integrate_kernel")
     else:
         # SM-local bound: shared-memory bandwidth, 32 banks x 4 B per clock per
         # SM at the SM clock sampled during the timed steps
@@ -923,11 +933,7 @@ def main():
         roof["dram_gbs"] = traffic / (kms / 1e3) / 1e9
         roof["dram_frac_of_hbm"] = roof["dram_gbs"] / peaks["hbm_gbs"]
         roof["hbm_peak_source"] = f"MEASURED_PEAKS.json hbm_gbs ({src})"
-    groups = None
-    if tuned:
-        groups = n_sms * (tuned["threads_per_cta"] // tuned["threads_per_zone"])
-    elif args.tpz and args.tpc:
-        groups = n_sms * (args.tpc // args.tpz)
+    groups = zones_in_flight(tb["zone_ns"]) if tuned or (args.tpz and args.tpc) else None
     dtype = {"mixed": "f32 (float-float state)", "mixed_fp64": "f32 fluxes, f64 update", "fp64": "f64",
              "qss_fp64": "f64", "qss_mixed": "f32 (float-float state)"}[args.form]
     line = {"metric": METRIC, "value": value, "unit": "zone-steps/s", "n_gpus": world, "steps": args.steps,
