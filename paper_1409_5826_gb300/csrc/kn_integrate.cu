@@ -5,9 +5,10 @@
 // Execution model (sm_103a):
 //   * one persistent launch; each CTA is split into M zone groups of G
 //     threads (G = CTA size: CTA-per-zone; G = 128: warp-group-per-zone);
-//   * every group pulls zones from its network's work queue (one atomic per
-//     zone, longest predicted zones first) and keeps the zone resident in
-//     shared memory for its whole integration;
+//   * every group starts with a zone dealt over the CTAs, then pulls zones from
+//     its network's work queue (one atomic per zone, longest predicted zones
+//     first), and keeps the zone resident in shared memory for its whole
+//     integration;
 //   * a network's tables (reactant lists, rate parameters, the sliced gather
 //     list) are staged once per CTA into shared memory and shared by all
 //     groups;

@@ -27,7 +27,7 @@
 // the terms of a piece, the segmented reduction, the butterflies, the warps), so
 // the results are the group kernel's bit for bit, whatever T and NZ.
 //
-// Measured against the group kernel: 4096 zones of 150/1604 to 1e-9 s 818 -> 648
+// Measured against the group kernel: 4096 zones of 150/1604 to 1e-9 s 818 -> 640
 // ms, 100 zones of it (one an SM) 7.2 -> 3.5 ms, 8001 zones of the 16/48 chain to
 // 1e-3 s 32.6 -> 20.5 ms, 1000 of 365/4400 to 3e-11 s 42.5 -> 37.3 ms, 4096 QSS
 // chains to 1e-2 s 56.9 -> 38.5 ms.
