@@ -269,11 +269,12 @@ static kn_status plan_slots(kn_network* const* nets, int n_nets, const Tiling* t
             // more threads step faster, 100 species 32 against 38 ms at two of 256 and
             // three of 160), each of at least the species' warps and the one that
             // decides, then all threads to those groups
-            const int lo = warp ? 32 : (n->N + 31) / 32 * 32 + 32;
-            const int most = std::max(1, std::min({warp ? kSlotThreads / 32 : 3, kSlotThreads / lo, (zps + NZ - 1) / NZ}));
+            const int lo = slot_min_threads(n, warp);
+            const int most = std::max(
+                1, std::min({warp ? kSlotThreads / 32 : kMaxSlotGroups, kSlotThreads / lo, (zps + NZ - 1) / NZ}));
             bool fit = false;
             auto try_plan = [&](int cap, int ng) -> kn_status {
-                const int T = warp ? 32 : kSlotThreads / ng / 32 * 32;
+                const int T = slot_threads(warp, ng);
                 if (T < lo) return KN_OK;
                 SlotBlob* sb;
                 kn_status s = get_slots(n, tl[p].G, T, NZ, cap, &sb);
@@ -379,9 +380,12 @@ kn_status kn_check_gather_tables(const kn_network_desc* d, int32_t precision, in
         SlotTables st;
         bool fits;
         for (int NZ = 1; NZ <= 2; ++NZ)
-            for (int W = warp ? 1 : (n->N + 31) / 32 + 1; W <= (warp ? 1 : kSlotThreads / 32); ++W)
-                for (int cap = warp ? kCapWarp : kCapGroup; cap <= (warp ? kCapWarp : kCapWide); ++cap)
-                    if ((s = build_slots_host(n.get(), T, 32 * W, NZ, cap, sb, st, fits)) != KN_OK) return s;
+            for (int ng = 1; ng <= (warp ? 1 : kMaxSlotGroups); ++ng)
+                for (int cap = warp ? kCapWarp : kCapGroup; cap <= (warp ? kCapWarp : kCapWide); ++cap) {
+                    const int t = slot_threads(warp, ng);
+                    if (t < slot_min_threads(n.get(), warp)) continue;
+                    if ((s = build_slots_host(n.get(), T, t, NZ, cap, sb, st, fits)) != KN_OK) return s;
+                }
     }
     stats[0] = T.L;
     stats[1] = T.n_slices;

@@ -62,6 +62,7 @@ struct Tables {
     std::unique_ptr<DevBuf> blob;
     TableLayout tl{};
     GatherOrder order;                               // mixed form
+    std::vector<int> banks;                          // kn_slots.cu: V's values' banks, found on first use
     std::map<std::pair<int, int>, SlotBlob> slots;   // (threads, 8 zones per group + capacities) -> device blob
     int L = 0, n_slices = 0, warp_len = 0;  // piece cap, slices, longest warp's terms per lane
 };
@@ -108,7 +109,12 @@ kn_status build_tables_host(const kn_network* n, int prec, int Q, std::vector<un
 // capacities kSlotCaps[cap], from the summation order of `tb`; checked on the host
 // like the tables.  fits = false: the network does not fit the capacities or the
 // 16-bit offsets.
-kn_status build_slots_host(const kn_network* n, const Tables& tb, int T, int NZ, int cap, std::vector<unsigned char>& blob,
+kn_status build_slots_host(const kn_network* n, Tables& tb, int T, int NZ, int cap, std::vector<unsigned char>& blob,
                            SlotTables& st, bool& fits);
+// kn_slots.cu: the threads of a group when a CTA holds ng of them, and the fewest that a
+// group needs: the species' warps and the one that decides.  One warp if the order is.
+constexpr int kMaxSlotGroups = 3;
+inline int slot_threads(bool warp, int ng) { return warp ? 32 : kSlotThreads / ng / 32 * 32; }
+inline int slot_min_threads(const kn_network* n, bool warp) { return warp ? 32 : (n->N + 31) / 32 * 32 + 32; }
 SlotLayout slot_layout(const kn_network* n, const SlotTables& st, int T, int NZ, bool qss);
 }  // namespace kn

@@ -484,9 +484,49 @@ static std::vector<int> place_banks(int nv, const std::vector<std::vector<int>>&
     }
     return bank;
 }
+
+// V's rows of 32 words, with room for the banks' search; the last holds the constant 0
+static int slot_rows(const kn_network* n) {
+    return (n->R + n->S_r + 31) / 32 + 1 + ((n->R + 31) / 32 > 4 ? 8 : 0);
+}
+
+// Banks for V's values, from the instructions that store and load them: the blocks of
+// 32 reactions and the gather's steps, whichever thread has them, so one search serves
+// every group size, number of zones and capacity of a summation order.
+static std::vector<int> slot_banks(const kn_network* n, const Tables& tb) {
+    const int R = n->R, blocks = (R + 31) / 32, zero_idx = R + n->S_r;
+    const int plane[3] = {R, 2 * R - n->R1, 3 * R - n->R1 - n->R12};
+    std::vector<std::vector<int>> groups;
+    std::vector<char> zero;
+    for (int b = 0; b < blocks; ++b)
+        for (int q = 0; q < 4; ++q) {
+            std::vector<int> g;
+            for (int j = 32 * b; j < std::min(R, 32 * b + 32); ++j) {
+                const int nr = n->nr[n->perm[j]];
+                if (q == 0) g.push_back(j);
+                else if (q <= nr && nr > 1) g.push_back(plane[q - 1] + j);  // (1-body partials: only at a refresh)
+            }
+            if (g.empty()) continue;
+            groups.push_back(std::move(g));
+            zero.push_back(0);
+        }
+    for (const auto& sl : tb.order.slices)
+        for (int k = 0; k < sl.len; ++k) {
+            std::vector<int> g;
+            char z = 0;
+            for (int l = 0; l < 32; ++l) {
+                const int v = sl.terms[32 * (size_t)k + l];
+                z |= v == zero_idx;
+                if (v != zero_idx && std::find(g.begin(), g.end(), v) == g.end()) g.push_back(v);
+            }
+            groups.push_back(std::move(g));
+            zero.push_back(z);
+        }
+    return place_banks(zero_idx, groups, zero, slot_rows(n) - 1);
+}
 }  // namespace
 
-kn_status build_slots_host(const kn_network* n, const Tables& tb, int T, int NZ, int cap, std::vector<unsigned char>& blob,
+kn_status build_slots_host(const kn_network* n, Tables& tb, int T, int NZ, int cap, std::vector<unsigned char>& blob,
                            SlotTables& st, bool& fits) {
     fits = false;
     st = SlotTables{};
@@ -556,41 +596,16 @@ kn_status build_slots_host(const kn_network* n, const Tables& tb, int T, int NZ,
         (to == 1 ? k1 : (to == 2 ? k2 : ka))[w].push_back(x.b);
         fl[w] += to == 3 ? 30 : x.cost;
     }
-    // ---- V: banks for the values, from the instructions that store and load them ----
+    // ---- V: the values' places, by their banks (slot_banks) ----
     const int plane[3] = {R, 2 * R - n->R1, 3 * R - n->R1 - n->R12};
-    std::vector<std::vector<int>> groups;
-    std::vector<char> zero;
-    for (int b = 0; b < blocks; ++b)
-        for (int q = 0; q < 4; ++q) {
-            std::vector<int> g;
-            for (int j = 32 * b; j < std::min(R, 32 * b + 32); ++j) {
-                const int nr = n->nr[n->perm[j]];
-                if (q == 0) g.push_back(j);
-                else if (q <= nr && nr > 1) g.push_back(plane[q - 1] + j);  // (1-body partials: only at a refresh)
-            }
-            if (g.empty()) continue;
-            groups.push_back(std::move(g));
-            zero.push_back(0);
-        }
-    for (const auto& sl : tb.order.slices)
-        for (int k = 0; k < sl.len; ++k) {
-            std::vector<int> g;
-            char z = 0;
-            for (int l = 0; l < 32; ++l) {
-                const int v = sl.terms[32 * (size_t)k + l];
-                z |= v == zero_idx;
-                if (v != zero_idx && std::find(g.begin(), g.end(), v) == g.end()) g.push_back(v);
-            }
-            groups.push_back(std::move(g));
-            zero.push_back(z);
-        }
-    st.vrows = (zero_idx + 31) / 32 + 1 + (blocks > 4 ? 8 : 0);  // with room for the banks' search
-    const std::vector<int> bank = place_banks(zero_idx, groups, zero, st.vrows - 1);
+    st.vrows = slot_rows(n);
+    if (32 * NZ * st.vrows > 0x10000) return KN_OK;
+    if (tb.banks.empty()) tb.banks = slot_banks(n, tb);
+    const std::vector<int>& bank = tb.banks;
     std::vector<int> at(zero_idx + 1), next(32, 0);
     for (int v = 0; v < zero_idx; ++v) at[v] = 32 * NZ * next[bank[v]]++ + bank[v];
     at[zero_idx] = 32 * NZ * (st.vrows - 1);
     st.zero = at[zero_idx];
-    if (32 * NZ * st.vrows > 0x10000) return KN_OK;
     // ---- the words ----
     st.slots = C.f1 + C.f2 + C.fa;
     const int nwords = C.f1 + 3 * C.f2 + 4 * C.fa + C.ga + C.gb + 3;
