@@ -306,7 +306,9 @@ kn_status kn_set_zone_conditions(kn_network *net, int32_t n_zones, const kn_zone
  * `stream`: results are in the networks' device state when the stream
  * reaches this point; read them with kn_get_abundances.  Results overwrite
  * the zone abundances in place, so a second call continues from them once
- * new conditions are set.  nets must be distinct.
+ * new conditions are set.  nets must be distinct.  The first call with a
+ * network at a precision and tiling builds its tables on the host, allocates
+ * and copies them; later ones, with any number of zones, only enqueue.
  * Errors: KN_ERR_INVALID_ARG (bad opts or tiling), KN_ERR_STATE (a network
  * without zones), KN_ERR_CUDA.
  */

@@ -66,6 +66,22 @@ static kn_status get_tables(kn_network* n, int prec, int Q, Tables** out) {
     return KN_OK;
 }
 
+// f(0) .. f(count - 1) on the host's threads; f throws nothing
+template <class F> static void side_by_side(size_t count, F f) {
+    std::atomic<size_t> next{0};
+    auto work = [&]() {
+        for (size_t i; (i = next.fetch_add(1)) < count;) f(i);
+    };
+    std::vector<std::thread> pool;
+    const size_t threads = std::min<size_t>(count, std::max(1u, std::thread::hardware_concurrency()));
+    try {
+        while (pool.size() + 1 < threads) pool.emplace_back(work);
+    } catch (const std::exception&) {  // no more threads: the ones there are do the work
+    }
+    work();
+    for (auto& t : pool) t.join();
+}
+
 // The tables of every group size G0, G0 + 32, .. G1, the missing ones built side by
 // side: a default launch looks at up to 12 of them (5 ms each for 150/1604).
 static kn_status build_tables_range(kn_network* n, int prec, int G0, int G1) {
@@ -80,26 +96,15 @@ static kn_status build_tables_range(kn_network* n, int prec, int G0, int G1) {
     for (int G = G0; G <= G1; G += 32)
         if (!n->tables.count({prec, G})) jobs.push_back({G, {}, {}, KN_OK, {}});
     if (jobs.size() < 2) return KN_OK;  // get_tables builds it
-    std::atomic<size_t> next{0};
-    auto work = [&]() {
-        for (size_t i; (i = next.fetch_add(1)) < jobs.size();) {
-            Job& j = jobs[i];
-            try {
-                j.s = build_tables_host(n, prec, j.G, j.blob, j.T);
-                if (j.s != KN_OK) j.msg = last_error();  // the message is this thread's
-            } catch (const std::exception&) {
-                j.s = KN_ERR_NOMEM;
-            }
+    side_by_side(jobs.size(), [&](size_t i) {
+        Job& j = jobs[i];
+        try {
+            j.s = build_tables_host(n, prec, j.G, j.blob, j.T);
+            if (j.s != KN_OK) j.msg = last_error();  // the message is this thread's
+        } catch (const std::exception&) {
+            j.s = KN_ERR_NOMEM;
         }
-    };
-    std::vector<std::thread> pool;
-    const size_t threads = std::min<size_t>(jobs.size(), std::max(1u, std::thread::hardware_concurrency()));
-    try {
-        while (pool.size() + 1 < threads) pool.emplace_back(work);
-    } catch (const std::exception&) {  // no more threads: the ones there are do the work
-    }
-    work();
-    for (auto& t : pool) t.join();
+    });
     for (Job& j : jobs) {
         if (j.s != KN_OK) return fail(j.s, "%s", j.msg.c_str());
         j.T.blob.reset(new DevBuf());
@@ -222,23 +227,63 @@ static kn_status plan_tiling(kn_network* n, int prec, int P, int budget, int G_f
     return KN_OK;
 }
 
-// The slot tables of one network for (G, T, NZ, cap), built on first use.
-static kn_status get_slots(kn_network* n, int G, int T, int NZ, int cap, SlotBlob** out) {
-    Tables& tb = n->tables.at({kPrecMixed, G});
-    auto it = tb.slots.find({T, 8 * NZ + cap});
-    if (it == tb.slots.end()) {
+// Every slot table that a summation order's launches can come to, built when the first
+// of them needs one: threads per group and zones per group follow from the number of
+// zones, and a call with another number of zones allocates and copies nothing.  The
+// first build searches the banks, the others then go side by side.
+static kn_status build_slots(kn_network* n, Tables& tb, bool warp, int budget) {
+    struct Job {
+        int T, NZ, cap;
         std::vector<unsigned char> blob;
-        SlotBlob sb;
-        kn_status s = build_slots_host(n, tb, T, NZ, cap, blob, sb.st, sb.fits);
-        if (s != KN_OK) return s;
-        if (sb.fits) {
-            sb.blob.reset(new DevBuf());
-            KN_CUDA(sb.blob->ensure(blob.size()));
-            KN_CUDA(cudaMemcpy(sb.blob->p, blob.data(), blob.size(), cudaMemcpyHostToDevice));
+        SlotTables st;
+        bool fits;
+        kn_status s;
+        std::string msg;
+    };
+    std::vector<Job> jobs;
+    auto build = [&](Job& j) {
+        try {
+            j.s = build_slots_host(n, tb, j.T, j.NZ, j.cap, j.blob, j.st, j.fits);
+            if (j.s != KN_OK) j.msg = last_error();  // the message is this thread's
+        } catch (const std::exception&) {
+            j.s = KN_ERR_NOMEM;
         }
-        it = tb.slots.emplace(std::make_pair(T, 8 * NZ + cap), std::move(sb)).first;
+    };
+    const int first = warp ? kCapWarp : kCapGroup, last = warp ? kCapWarp : kCapWide;
+    std::vector<Job> more;
+    for (int NZ = 1; NZ <= 2; ++NZ)
+        for (int cap = first; cap <= last; ++cap) {
+            // the largest group first: where it fits, plan_slots takes no later capacities
+            Job j{slot_threads(warp, 1), NZ, cap, {}, {}, false, KN_OK, {}};
+            if (j.T < slot_min_threads(n, warp)) continue;
+            build(j);
+            const bool enough = j.fits && j.st.bytes + slot_layout(n, j.st, j.T, NZ, true).bytes <= budget;
+            jobs.push_back(std::move(j));
+            for (int ng = 2; ng <= (warp ? 1 : kMaxSlotGroups); ++ng)
+                if (slot_threads(warp, ng) >= slot_min_threads(n, warp))
+                    more.push_back({slot_threads(warp, ng), NZ, cap, {}, {}, false, KN_OK, {}});
+            if (enough) break;
+        }
+    if (!tb.banks.empty()) side_by_side(more.size(), [&](size_t i) { build(more[i]); });
+    else for (Job& j : more) build(j);  // none of the first came to the search
+    for (Job& j : more) jobs.push_back(std::move(j));
+    std::vector<unsigned char> all;
+    std::vector<size_t> at;
+    for (Job& j : jobs) {
+        if (j.s != KN_OK) return fail(j.s, "%s", j.msg.c_str());
+        at.push_back(all.size());
+        if (j.fits) all.insert(all.end(), j.blob.begin(), j.blob.end());
+        all.resize((all.size() + 255) / 256 * 256);
     }
-    *out = &it->second;
+    tb.slot_blob.reset(new DevBuf());
+    if (!all.empty()) {
+        KN_CUDA(tb.slot_blob->ensure(all.size()));
+        KN_CUDA(cudaMemcpy(tb.slot_blob->p, all.data(), all.size(), cudaMemcpyHostToDevice));
+    }
+    for (size_t i = 0; i < jobs.size(); ++i)
+        tb.slots[{jobs[i].T, 8 * jobs[i].NZ + jobs[i].cap}] =
+            SlotBlob{tb.slot_blob->as<unsigned char>() + at[i], jobs[i].st, jobs[i].fits};
+    tb.slots_built = true;
     return KN_OK;
 }
 
@@ -265,6 +310,11 @@ static kn_status plan_slots(kn_network* const* nets, int n_nets, const Tiling* t
             PlanDev& P = lp.plans[p];
             const bool warp = tl[p].G == 32;
             if (warp && !rate_cache_on(n, kPrecMixed)) return KN_OK;
+            Tables& tb = n->tables.at({kPrecMixed, tl[p].G});
+            if (!tb.slots_built) {
+                const kn_status s = build_slots(n, tb, warp, budget);
+                if (s != KN_OK) return s;
+            }
             // the most groups that the zones can use (three at most: fewer groups of
             // more threads step faster, 100 species 32 against 38 ms at two of 256 and
             // three of 160), each of at least the species' warps and the one that
@@ -273,30 +323,25 @@ static kn_status plan_slots(kn_network* const* nets, int n_nets, const Tiling* t
             const int most = std::max(
                 1, std::min({warp ? kSlotThreads / 32 : kMaxSlotGroups, kSlotThreads / lo, (zps + NZ - 1) / NZ}));
             bool fit = false;
-            auto try_plan = [&](int cap, int ng) -> kn_status {
+            auto try_plan = [&](int cap, int ng) {
                 const int T = slot_threads(warp, ng);
-                if (T < lo) return KN_OK;
-                SlotBlob* sb;
-                kn_status s = get_slots(n, tl[p].G, T, NZ, cap, &sb);
-                if (s != KN_OK || !sb->fits) return s;
-                const SlotLayout sl = slot_layout(n, sb->st, T, NZ, qss);
-                if (sb->st.bytes + ng * sl.bytes > budget) return KN_OK;
-                P.slot_blob = (const unsigned char*)sb->blob->p;
-                P.st = sb->st;
+                const auto sb = tb.slots.find({T, 8 * NZ + cap});
+                if (sb == tb.slots.end() || !sb->second.fits) return;
+                const SlotTables& st = sb->second.st;
+                const SlotLayout sl = slot_layout(n, st, T, NZ, qss);
+                if (st.bytes + ng * sl.bytes > budget) return;
+                P.slot_blob = sb->second.blob;
+                P.st = st;
                 P.sl = sl;
                 P.T = T;
                 P.ng = ng;
                 P.cap = cap;
                 fit = true;
-                bytes = std::max(bytes, P.st.bytes + ng * sl.bytes);
+                bytes = std::max(bytes, st.bytes + ng * sl.bytes);
                 threads = std::max(threads, ng * T);
-                return KN_OK;
             };
             for (int cap = warp ? kCapWarp : kCapGroup; cap <= (warp ? kCapWarp : kCapWide) && !fit; ++cap)
-                for (int ng = most; ng >= 1 && !fit; --ng) {
-                    const kn_status s = try_plan(cap, ng);
-                    if (s != KN_OK) return s;
-                }
+                for (int ng = most; ng >= 1 && !fit; --ng) try_plan(cap, ng);
             all = fit;
         }
         if (!all) continue;

@@ -52,8 +52,9 @@ struct GatherOrder {
     std::vector<Slice> slices;
 };
 
+// one of an order's slot tables; blob points into Tables::slot_blob
 struct SlotBlob {
-    std::unique_ptr<DevBuf> blob;
+    const unsigned char* blob = nullptr;
     SlotTables st{};
     bool fits = false;
 };
@@ -63,7 +64,9 @@ struct Tables {
     TableLayout tl{};
     GatherOrder order;                               // mixed form
     std::vector<int> banks;                          // kn_slots.cu: V's values' banks, found on first use
-    std::map<std::pair<int, int>, SlotBlob> slots;   // (threads, 8 zones per group + capacities) -> device blob
+    std::map<std::pair<int, int>, SlotBlob> slots;   // (threads, 8 zones per group + capacities) -> table
+    std::unique_ptr<DevBuf> slot_blob;
+    bool slots_built = false;
     int L = 0, n_slices = 0, warp_len = 0;  // piece cap, slices, longest warp's terms per lane
 };
 }  // namespace kn
