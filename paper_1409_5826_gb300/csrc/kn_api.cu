@@ -435,7 +435,7 @@ kn_status kn_check_gather_tables(const kn_network_desc* d, int32_t precision, in
     stats[0] = T.L;
     stats[1] = T.n_slices;
     stats[2] = T.warp_len;
-    stats[3] = (int)blob.size();
+    stats[3] = T.tl.bytes;
     return KN_OK;
 }
 
@@ -788,10 +788,11 @@ static kn_status prepare_launch(kn_network* const* nets, int n_nets, const kn_op
         }
         const int W = prec == kPrecFP64 && need <= 2 ? wide_group(P.G) : 0;
         const GroupLayout gl = group_layout(nets[0], prec, W, extras);
-        const int bytes = (P.smem_tables ? P.tl.bytes : 0) + P.M * gl.bytes;
+        const int bytes = (P.smem_tables ? P.tl.wide_bytes : 0) + P.M * gl.bytes;
         if (W > P.G && P.G >= 64 && P.N <= P.G && P.M * W <= 1024 && P.M * P.G == P_best && bytes <= budget) {
             P.G = W;
             P.wide = 1;
+            P.tl.bytes = P.tl.wide_bytes;
             P.gl = gl;
             P_best = P.M * W;
             max_smem = std::max(max_smem, bytes);

@@ -44,7 +44,7 @@ constexpr int kMlpSmemBytes = (kMlpFeatures * kMlpHidden + kMlpHidden * kMlpHidd
 // Reactions are stored sorted by reactant count (1-body, 2-body, 3-body) so
 // that the flux loop is warp-uniform and multiplies by no sentinel.
 struct TableLayout {
-    int32_t bytes;        // total (multiple of 16)
+    int32_t bytes;        // staged in shared memory (multiple of 16)
     int32_t off_A;        // mass numbers (integers, exact): float[N] in the mixed form, double[N] in the
                           //   forms with an FP64 update
     int32_t off_rspec;    // uint32[R]: reactant species a | b << 10 | c << 20 (N = none)
@@ -56,7 +56,7 @@ struct TableLayout {
     int32_t off_sidx;     // uint16[sum_s 32 len_s]: terms, lane-interleaved: byte offsets into V
                           //   when sidx_bytes, else V indices
     int32_t sidx_bytes;   // 1: sidx holds byte offsets
-    int32_t n_slices;
+    int32_t wide_bytes;   // FP64 form, wide groups: the bytes staged, with the list at off_deal (= bytes)
     int32_t off_deal;     // FP64 form: the slices dealt to wide_group(G) / 32 warps: uint16 ranges
                           //   [warps + 1] into the slice numbers [n_slices] that follow
 };

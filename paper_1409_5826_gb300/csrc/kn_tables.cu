@@ -328,8 +328,7 @@ kn_status build_tables_host(const kn_network* n, int prec, int Q, std::vector<un
     // the slices dealt to a wide group's warps, longest first: to the scheduler (w mod 4)
     // with the least to do, and there to the warp with the least
     std::vector<uint16_t> deal;
-    tl.n_slices = n_slices;
-    tl.off_deal = off;
+    tl.bytes = tl.off_deal = off;
     if (prec == kPrecFP64) {
         const int D = wide_group(G) / 32;
         std::vector<int> by(n_slices), load(D, 0), sched(4, 0);
@@ -350,7 +349,7 @@ kn_status build_tables_host(const kn_network* n, int prec, int Q, std::vector<un
         for (auto& m : mine) deal.insert(deal.end(), m.begin(), m.end());
         off = pad16(off + 2 * (int)deal.size());
     }
-    tl.bytes = off;
+    tl.wide_bytes = off;
     blob.assign(off, 0);
     for (int i = 0; i < N; ++i) {
         if (a_bytes == 8) {
