@@ -616,7 +616,9 @@ static void set_guard_band(OptsDev& D, const kn_opts* o) {
                o->safety * o->eps_r >= 1e-25 && o->safety * o->eps_c >= 1e-25 &&
                o->grow_max < 1e29 * o->safety * std::min(o->eps_r, o->eps_c);
     D.shrink32 = (float)o->shrink;
-    D.dt_min32 = (float)o->dt_min_frac;
+    // kn_slots.cu compares in FP64 below 4 dt_min32 t: a fraction below the FP32 range
+    // must not become 0
+    D.dt_min32 = o->dt_min_frac > 0 ? std::max((float)o->dt_min_frac, 1.17549435e-38f) : 0.f;
     D.band_lo32 = (float)(1.0 - band);
     D.band_hi32 = (float)(1.0 + band);
     D.thr_lo32 = (float)(o->eps_r * (1.0 - band));
