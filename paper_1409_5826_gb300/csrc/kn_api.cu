@@ -48,8 +48,7 @@ static kn_status build_tables(kn_network* n, int prec, int Q, Tables& T) {
     kn_status s = build_tables_host(n, prec, Q, blob, T);
     if (s != KN_OK) return s;
     T.blob.reset(new DevBuf());
-    KN_CUDA(T.blob->ensure(blob.size()));
-    KN_CUDA(cudaMemcpy(T.blob->p, blob.data(), blob.size(), cudaMemcpyHostToDevice));
+    KN_CUDA(T.blob->upload(blob.data(), blob.size()));
     return KN_OK;
 }
 
@@ -108,8 +107,7 @@ static kn_status build_tables_range(kn_network* n, int prec, int G0, int G1) {
     for (Job& j : jobs) {
         if (j.s != KN_OK) return fail(j.s, "%s", j.msg.c_str());
         j.T.blob.reset(new DevBuf());
-        KN_CUDA(j.T.blob->ensure(j.blob.size()));
-        KN_CUDA(cudaMemcpy(j.T.blob->p, j.blob.data(), j.blob.size(), cudaMemcpyHostToDevice));
+        KN_CUDA(j.T.blob->upload(j.blob.data(), j.blob.size()));
         n->tables.emplace(std::make_pair(prec, j.G), std::move(j.T));
     }
     return KN_OK;
@@ -276,10 +274,7 @@ static kn_status build_slots(kn_network* n, Tables& tb, bool warp, int budget) {
         all.resize((all.size() + 255) / 256 * 256);
     }
     tb.slot_blob.reset(new DevBuf());
-    if (!all.empty()) {
-        KN_CUDA(tb.slot_blob->ensure(all.size()));
-        KN_CUDA(cudaMemcpy(tb.slot_blob->p, all.data(), all.size(), cudaMemcpyHostToDevice));
-    }
+    if (!all.empty()) KN_CUDA(tb.slot_blob->upload(all.data(), all.size()));
     for (size_t i = 0; i < jobs.size(); ++i)
         tb.slots[{jobs[i].T, 8 * jobs[i].NZ + jobs[i].cap}] =
             SlotBlob{tb.slot_blob->as<unsigned char>() + at[i], jobs[i].st, jobs[i].fits};
@@ -396,8 +391,7 @@ kn_status kn_create_network(const kn_network_desc* d, kn_network** out) {
     std::vector<double> r0;
     kn_status s = network_host_setup(d, n, r0);
     if (s != KN_OK) return s;
-    KN_CUDA(n->rate0.ensure(8 * r0.size()));
-    KN_CUDA(cudaMemcpy(n->rate0.p, r0.data(), 8 * r0.size(), cudaMemcpyHostToDevice));
+    KN_CUDA(n->rate0.upload(r0.data(), 8 * r0.size()));
     KN_CUDA(n->qhead.ensure(64));
     *out = n.release();
     return KN_OK;
@@ -1344,8 +1338,7 @@ kn_status kn_set_binding_energies(kn_network* n, const double* B) {
     if (!n || !B) return fail(KN_ERR_INVALID_ARG, "kn_set_binding_energies: NULL argument");
     for (int i = 0; i < n->N; ++i)
         if (!std::isfinite(B[i])) return fail(KN_ERR_INVALID_ARG, "kn_set_binding_energies: B[%d] not finite", i);
-    KN_CUDA(n->bind.ensure(8 * (size_t)n->N));
-    KN_CUDA(cudaMemcpy(n->bind.p, B, 8 * (size_t)n->N, cudaMemcpyHostToDevice));
+    KN_CUDA(n->bind.upload(B, 8 * (size_t)n->N));
     n->has_bind = true;
     return KN_OK;
 }

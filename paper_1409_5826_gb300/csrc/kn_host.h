@@ -39,6 +39,15 @@ struct DevBuf {
         if (e == cudaSuccess) bytes = b;
         return e;
     }
+    // Grow to b bytes and copy them from pageable host memory.  Such a copy may return
+    // with its last part still on the way, ordered before later work on streams that
+    // follow the default stream only; after the wait it is there for every stream.
+    cudaError_t upload(const void* src, size_t b) {
+        cudaError_t e = ensure(b);
+        if (e == cudaSuccess) e = cudaMemcpy(p, src, b, cudaMemcpyHostToDevice);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
+        return e;
+    }
     template <class T> T* as() const { return (T*)p; }
 };
 

@@ -436,6 +436,7 @@ kn_status kn_mlp_create(kn_mlp** out) {
         for (int k = 0; k < NF; ++k) nm[NF + k] = 1.f;
         e = cudaMemcpy(m->norm, nm.data(), sizeof(float) * 2 * NF, cudaMemcpyHostToDevice);
     }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);  // for calls on any stream
     if (e != cudaSuccess) {
         kn_mlp_destroy(m);
         return cuda_fail(e);

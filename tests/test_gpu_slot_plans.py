@@ -60,3 +60,25 @@ def test_another_number_of_zones_under_capture(env, net, most, zones):
         assert (r["status"] == 0).all()
         del graph
     g.close()
+
+
+@pytest.mark.parametrize("prec", [0, 1, 2])
+def test_first_launch_on_a_stream_of_its_own(env, prec):
+    """A network's tables are on the device before its first launch on a stream that does
+    not follow the default stream: the same bits as a launch that finds them there."""
+    torch, kn = env
+    net = net150()
+    dz = _device(torch, profile_zones(net, 40, base_seed=43, t_end=3e-12))
+    torch.cuda.synchronize()
+    s = torch.cuda.Stream()
+    for rep in range(4):
+        g = kn.Network(net)
+        g.set_binding_energies(np.linspace(1.0, 2.0, net.n_species))
+        runs = []
+        for _ in range(2):
+            g.set_zones(dz, s)
+            kn.integrate_batch([g], kn.Opts(precision=prec), s)
+            runs.append({**g.get(s), "E": g.energy(s)})
+        for k in OUT + ("E",):
+            assert np.array_equal(runs[0][k], runs[1][k]), k
+        g.close()
