@@ -315,6 +315,28 @@ kn_status kn_set_zone_conditions(kn_network *net, int32_t n_zones, const kn_zone
 kn_status kn_integrate_batch(kn_network *const *nets, int32_t n_nets, const kn_opts *opts,
                              void *stream);
 
+/* The kernel and tiling of a network's last kn_integrate_batch. */
+enum {
+    KN_KERNEL_GROUP = 0, /* a thread group per zone */
+    KN_KERNEL_SLOTS = 1  /* KN_PREC_MIXED: one or two zones per thread group */
+};
+typedef struct {
+    int32_t kernel;            /* KN_KERNEL_* */
+    int32_t threads_per_zone;  /* the order of the sums: the same value in kn_opts gives the same bits */
+    int32_t threads_per_group; /* threads of a group as launched */
+    int32_t zones_per_group;   /* 1 or 2 */
+    int32_t groups_per_cta;
+    int32_t ctas;              /* CTAs that begin with this network's zones */
+} kn_launch_info;
+
+/*
+ * What the last kn_integrate_batch with `net` launched (host state, no device
+ * work): which kernel took the network and the zone slots that it gave it,
+ * ctas x groups_per_cta x zones_per_group.
+ * Errors: KN_ERR_INVALID_ARG (NULL), KN_ERR_STATE (no such call yet).
+ */
+kn_status kn_get_launch_info(const kn_network *net, kn_launch_info *info);
+
 /*
  * Copy results out (Sec. 6, step 3: abundances and the final dt, plus
  * per-zone counters).  Synchronises `stream` first.  Any output pointer may

@@ -832,6 +832,10 @@ static kn_status prepare_launch(kn_network* const* nets, int n_nets, const kn_op
         lp.plans[p].cta_end = b + cnt;
         lp.plans[p].dealt = cnt * (slots ? lp.plans[p].ng * lp.nz : lp.plans[p].M);
         b += cnt;
+        const PlanDev& L = lp.plans[p];
+        if (!probe)
+            nets[p]->launched = slots ? kn_launch_info{KN_KERNEL_SLOTS, tl[p].G, L.T, lp.nz, L.ng, cnt}
+                                      : kn_launch_info{KN_KERNEL_GROUP, tl[p].G, L.G, 1, L.M, cnt};
     }
     OptsDev& D = lp.o;
     D.kappa = o->kappa;
@@ -934,6 +938,13 @@ kn_status kn_integrate_batch(kn_network* const* nets, int32_t n_nets, const kn_o
         it = g_graphs.emplace(key, ge).first;
     }
     KN_CUDA(cudaGraphLaunch(it->second.x, st));
+    return KN_OK;
+}
+
+kn_status kn_get_launch_info(const kn_network* n, kn_launch_info* info) {
+    if (!n || !info) return fail(KN_ERR_INVALID_ARG, "kn_get_launch_info: NULL argument");
+    if (n->launched.kernel < 0) return fail(KN_ERR_STATE, "kn_get_launch_info: no kn_integrate_batch yet");
+    *info = n->launched;
     return KN_OK;
 }
 

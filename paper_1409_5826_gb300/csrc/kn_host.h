@@ -109,6 +109,7 @@ struct kn_network {
     int trial_Z = 0;        // > 0 during autotune trials: integrate only the first trial_Z zones of the queue
     int tuned_P[3][3] = {};  // [precision][plain, learned, QSS]: autotuned CTA size
     int tuned_G[3][3] = {};  // ... and zone group size
+    kn_launch_info launched = {-1, 0, 0, 0, 0, 0};  // the last kn_integrate_batch (kernel < 0: none yet)
 };
 
 namespace kn {

@@ -23,6 +23,7 @@ ZONE_STATUS = {0: "ok", 1: "step_limit", 2: "dt_underflow", 3: "nonfinite", 4: "
                5: "invalid", 6: "pending"}
 PREC_FP64, PREC_MIXED, PREC_MIXED_FP64 = 0, 1, 2
 METHOD_ASYMPTOTIC, METHOD_QSS = 0, 1
+KERNEL_GROUP, KERNEL_SLOTS = 0, 1
 MEM_HOST, MEM_DEVICE = 0, 1
 
 
@@ -67,6 +68,11 @@ class _Tiling(C.Structure):
                 ("zone_steps_per_s", C.c_double), ("candidates", C.c_int32), ("pad", C.c_int32)]
 
 
+class _LaunchInfo(C.Structure):
+    _fields_ = [(n, C.c_int32) for n in ("kernel", "threads_per_zone", "threads_per_group", "zones_per_group",
+                                         "groups_per_cta", "ctas")]
+
+
 _lib = None
 
 
@@ -89,6 +95,7 @@ def lib():
         "kn_check_gather_tables": (I32, [C.POINTER(_Desc), I32, I32, P]),
         "kn_set_zone_conditions": (I32, [P, I32, C.POINTER(_Zones), I32, P]),
         "kn_integrate_batch": (I32, [P, I32, C.POINTER(_Opts), P]),
+        "kn_get_launch_info": (I32, [P, C.POINTER(_LaunchInfo)]),
         "kn_get_abundances": (I32, [P, P, P, P, P, P, P, I32, P]),
         "kn_get_batch_stats": (I32, [P, I32, P, C.POINTER(_Stats)]),
         "kn_probe_step": (I32, [P, C.POINTER(_Opts), P, P, P, P, P, P]),
@@ -274,6 +281,12 @@ class Network:
         ptrs = [out[k].data_ptr() if k in out else None for k in keys]
         _check(lib().kn_get_abundances(self.h, *ptrs, MEM_DEVICE, C.c_void_p(_stream_ptr(stream))))
         return out
+
+    def launch_info(self) -> dict:
+        """The kernel and tiling of the network's last integrate_batch (kn_launch_info)."""
+        v = _LaunchInfo()
+        _check(lib().kn_get_launch_info(self.h, C.byref(v)))
+        return {f: getattr(v, f) for f, _ in _LaunchInfo._fields_}
 
     def advance(self, T9, rho, t_end, stream=None):
         """Operator splitting: continue every zone into the next hydro interval at

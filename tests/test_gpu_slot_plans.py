@@ -1,9 +1,13 @@
-"""The launches of the kernel with several zones per thread group: a network's first
-launch prepares what its launches with any number of zones need."""
+"""The launches of the kernel with several zones per thread group: which networks it
+takes (kn_get_launch_info); several networks in one launch, bit for bit against the
+group kernel; and that a network's first launch prepares what its launches with any
+number of zones need."""
+import ctypes as C
+
 import numpy as np
 import pytest
 
-from kn_inputs import chain_network, net150, net365, profile_zones
+from kn_inputs import chain_network, net150, net365, profile_zones, random_tiny_network, sweep_network
 
 pytestmark = pytest.mark.gpu
 IN = ("Y0", "T0", "rho0", "tau", "t_start", "t_end", "dt_trial")
@@ -81,4 +85,87 @@ def test_first_launch_on_a_stream_of_its_own(env, prec):
             runs.append({**g.get(s), "E": g.energy(s)})
         for k in OUT + ("E",):
             assert np.array_equal(runs[0][k], runs[1][k]), k
+        g.close()
+
+
+# the networks and orders that test_gpu_slots compares, and the kernel that each is to run
+@pytest.mark.parametrize("net,G,zones,kernel,per_group", [
+    (chain_network, 32, 1, 1, 1), (chain_network, 32, 5001, 1, 2), (lambda: sweep_network(32), 128, 153, 1, 1),
+    (lambda: sweep_network(64), 192, 304, 1, 1), (lambda: sweep_network(100), 160, 457, 1, 2),
+    (net150, 192, 1, 1, 1), (net150, 192, 611, 1, 2), (net150, 160, 1301, 1, 2),
+    (lambda: sweep_network(250), 320, 305, 1, 2), (net365, 512, 307, 1, 2), (net150, 128, 7, 0, 1),
+    (lambda: random_tiny_network(7, 11, 1), 32, 4, 1, 1), (lambda: random_tiny_network(10, 16, 2), 64, 4, 1, 1),
+])
+def test_the_kernel_that_runs(env, net, G, zones, kernel, per_group):
+    torch, kn = env
+    net = net()
+    opts = kn.Opts(precision=kn.PREC_MIXED, threads_per_zone=G, threads_per_cta=G, max_steps=20)
+    g = kn.Network(net)
+    with pytest.raises(kn.KnError) as e:
+        g.launch_info()
+    assert e.value.code == kn.KN_ERR_STATE
+    g.set_zones(_device(torch, profile_zones(net, zones, base_seed=31, t_end=3e-12)))
+    kn.integrate_batch([g], opts)
+    i = g.launch_info()
+    assert (i["kernel"], i["threads_per_zone"], i["zones_per_group"]) == (kernel, G, per_group)
+    assert i["groups_per_cta"] * i["threads_per_group"] <= 1024 and i["ctas"] >= 1
+    g.get()
+    # replay and records run the group kernel
+    if kernel:
+        feat = torch.zeros((1, 64), dtype=torch.float32, device="cuda")
+        lab = torch.zeros(1, dtype=torch.float32, device="cuda")
+        cnt = torch.zeros(1, dtype=torch.int64, device="cuda")
+        g.set_zones(_device(torch, profile_zones(net, 1, base_seed=31, t_end=3e-12)))
+        kn.integrate_batch([g], kn.Opts(precision=kn.PREC_MIXED, threads_per_zone=G, threads_per_cta=G, max_steps=2,
+                                        record_features=feat.data_ptr(), record_labels=lab.data_ptr(),
+                                        record_capacity=1, record_count=cnt.data_ptr()))
+        assert g.launch_info()["kernel"] == 0
+        g.get()
+    g.close()
+
+
+def _group_kernel(torch, kn, g, dz, opts):
+    """kn_integrate_noalloc: the group kernel on the same zones."""
+    Z = dz["T0"].shape[0]
+    f64 = dict(dtype=torch.float64, device="cuda")
+    out = {"Y": torch.empty((Z, g.N), **f64), "t": torch.empty(Z, **f64), "dt_next": torch.empty(Z, **f64),
+           "steps": torch.empty(Z, dtype=torch.int64, device="cuda"),
+           "rejects": torch.empty(Z, dtype=torch.int64, device="cuda"),
+           "status": torch.empty(Z, dtype=torch.int32, device="cuda")}
+    zc = kn._Zones(*[dz[k].data_ptr() for k in IN])
+    rc = kn.lib().kn_integrate_noalloc(g.h, Z, C.byref(zc), C.byref(opts.c()), *[out[k].data_ptr() for k in OUT],
+                                       C.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert rc == kn.KN_OK, kn.lib().kn_last_error()
+    torch.cuda.synchronize()
+    return {k: v.cpu().numpy() for k, v in out.items()}
+
+
+# CTAs of 480 threads give the 16-species chain one-warp groups, 64 and 150 species
+# groups of 160 threads and 365 species one of 480: a mix of all capacities.
+# (1, 0, 900): the chain's share of the CTAs rounds to none.
+@pytest.mark.parametrize("zones", [(1, 1, 1, 1), (2, 40, 1, 0), (1, 0, 900, 0), (700, 3, 160, 0), (0, 310, 5, 90),
+                                   (5000, 200, 33, 0), (40, 500, 60, 300), (0, 700, 0, 2)])
+@pytest.mark.parametrize("method", [0, 1])
+def test_several_networks_against_the_group_kernel(env, zones, method):
+    torch, kn = env
+    cta, order = 480, {16: 32, 64: 160, 150: 160, 365: 480}
+    gs, dzs = [], []
+    for net, Z in zip((chain_network(), net150(), net365(), sweep_network(64)), zones):
+        if Z:
+            gs.append(kn.Network(net))
+            dzs.append(_device(torch, profile_zones(net, Z, base_seed=44, t_end=3e-12)))
+            gs[-1].set_zones(dzs[-1])
+    opts = dict(precision=kn.PREC_MIXED, method=method, max_steps=20000)
+    kn.integrate_batch(gs, kn.Opts(threads_per_cta=cta, **opts))
+    for g, dz in zip(gs, dzs):
+        i = g.launch_info()
+        assert (i["kernel"], i["threads_per_zone"]) == (kn.KERNEL_SLOTS, order[g.N])
+        a = g.get()
+        G = order[g.N]
+        b = _group_kernel(torch, kn, g, dz, kn.Opts(threads_per_zone=G, threads_per_cta=G, **opts))
+        for k in OUT:
+            assert np.array_equal(a[k], b[k]), (g.N, k)
+        assert method or (a["status"] == 0).all()
+    assert zones != (1, 0, 900, 0) or gs[0].launch_info()["ctas"] == 0
+    for g in gs:
         g.close()
