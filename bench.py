@@ -396,12 +396,12 @@ def timed_batches(kn, nets, set_zones, opts, steps, warmup, stream, flush, zone_
             "zone_ns": zone_ns.cpu().numpy() if zone_ns is not None else None}
 
 
-def zones_in_flight(zone_ns):
-    """The most zones that were in the kernel's slots at one time (a thread group
-    holds one zone or two)."""
-    start, end = np.sort(zone_ns[:, 0]), np.sort(zone_ns[:, 1])
-    # zones that start at or after another's end may take its slot
-    return int((np.arange(1, len(start) + 1) - np.searchsorted(end, start, side="right")).max())
+KERNELS = {0: "integrate_kernel", 1: "slots_kernel"}
+
+
+def zone_slots(info):
+    """The zones that the launch has room for at one time (kn_launch_info)."""
+    return info["ctas"] * info["groups_per_cta"] * info["zones_per_group"]
 
 
 def tail_stats(zone_ns, steps, groups):
@@ -427,7 +427,7 @@ def _mean(x):
     return float(np.mean(x))
 
 
-def smem_roofline(parts, kms, clk, n_sms, qss=False, kernel="slots_kernel"):
+def smem_roofline(parts, kms, clk, n_sms, qss=False, kernel=None):
     """Shared-memory roofline of the FP32-flux forms: the measurement plan's
     bytes per accepted zone-step (algorithmic_smem_bytes, FP32 widths) over
     the kernel time, against 128 B/clk/SM x SMs x the sampled SM clock.
@@ -470,7 +470,8 @@ def _form_line(tb, nets, zones_total, roof, extra=None):
     out = {"zone_steps_per_s": st["steps"] / (kms / 1e3), "zones_per_s": st["zones_ok"] / (kms / 1e3),
            "ms_per_batch": _mean(tb["step_ms"]), "kernel_ms": kms, "kernel_ms_all": tb["kernel_ms"],
            "accepted_steps": st["steps"], "rejects": st["rejects"], "zones": zones_total,
-           "zones_ok": st["zones_ok"], "clocks": tb["clocks"], "roofline": roof}
+           "zones_ok": st["zones_ok"], "clocks": tb["clocks"], "roofline": roof,
+           "launch": [g.launch_info() for g in nets]}
     if extra:
         out.update(extra)
     return out
@@ -506,8 +507,11 @@ def other_forms(kn, g, net, zones, dz, stream, flush, mixed_line, args):
 
     zns = torch.zeros((zones.n_zones, 2), dtype=torch.int64, device=torch.device("cuda", torch.cuda.current_device()))
 
-    def tail_of(tb, tuned):
-        return tail_stats(tb["zone_ns"], g.get(stream)["steps"], zones_in_flight(tb["zone_ns"]) if tuned else None)
+    def tail_of(tb):
+        return tail_stats(tb["zone_ns"], g.get(stream)["steps"], zone_slots(g.launch_info()))
+
+    def kernel_of():
+        return KERNELS[g.launch_info()["kernel"]]
 
     out["mixed"] = {"median_rel_err_vs_tight_oracle": err(), "see": "the headline value and roofline"}
     # the split the measurement plan names: FP32 rates, fluxes and Kahan
@@ -523,10 +527,10 @@ def other_forms(kn, g, net, zones, dz, stream, flush, mixed_line, args):
     roof = fp64_roofline(update_fp64_flops(net, st["steps"] + st["rejects"]), kms, fp64_peak,
                          "11 FP64 operations per species per attempt (update, conservation sum, test)")
     roof["smem"] = smem_roofline([(net, st["steps"], st["rejects"])], kms, tb["clocks"], n_sms,
-                                 kernel="integrate_kernel")
+                                 kernel=kernel_of())
     out["mixed_fp64_update"] = _form_line(tb, [g], zones.n_zones, roof,
                                           {"median_rel_err_vs_tight_oracle": err(), "tiling": tuned,
-                                           "tail": tail_of(tb, tuned)})
+                                           "tail": tail_of(tb)})
     # every step in FP64
     g.set_zones(dz, stream)
     tuned = kn.autotune([g], kn.Opts(precision=kn.PREC_FP64), max_steps=100, stream=stream)
@@ -536,7 +540,7 @@ def other_forms(kn, g, net, zones, dz, stream, flush, mixed_line, args):
                          "rates 5 R + fluxes 1/3/7 per 1/2/3-body reaction + gathers S_r + S_p per accepted step, "
                          "11 N per attempt")
     out["fp64"] = _form_line(tb, [g], zones.n_zones, roof, {"median_rel_err_vs_tight_oracle": err(), "tiling": tuned,
-                                                            "tail": tail_of(tb, tuned)})
+                                                            "tail": tail_of(tb)})
     # the alpha-QSS update in FP64 (Sec. 11's question: does QSS in place of
     # Eq. 3 integrate faster on the GPU?); the same accept test and controller
     g.set_zones(dz, stream)
@@ -548,7 +552,7 @@ def other_forms(kn, g, net, zones, dz, stream, flush, mixed_line, args):
                          "rates 5 R + fluxes 1/3/7 per 1/2/3-body reaction + gathers S_r + S_p per accepted step "
                          "and again per attempt (the predicted state), 49 N per attempt")
     out["qss_fp64"] = _form_line(tb, [g], zones.n_zones, roof, {"median_rel_err_vs_tight_oracle": err(),
-                                                                "tiling": tuned, "tail": tail_of(tb, tuned)})
+                                                                "tiling": tuned, "tail": tail_of(tb)})
     out["qss_vs_asymptotic_fp64_zones_per_s"] = out["qss_fp64"]["zones_per_s"] / out["fp64"]["zones_per_s"]
     # the same in the mixed form, against the headline
     g.set_zones(dz, stream)
@@ -557,9 +561,9 @@ def other_forms(kn, g, net, zones, dz, stream, flush, mixed_line, args):
     tb = timed_batches(kn, [g], set_main, kn.Opts(**qo, use_graph=1), 3, 3, stream, flush, zns)
     st = tb["stats"]
     roof = smem_roofline([(net, st["steps"], st["rejects"])], _mean(tb["kernel_ms"]), tb["clocks"], n_sms,
-                         qss=True)
+                         qss=True, kernel=kernel_of())
     out["qss_mixed"] = _form_line(tb, [g], zones.n_zones, roof, {"median_rel_err_vs_tight_oracle": err(),
-                                                                 "tiling": tuned, "tail": tail_of(tb, tuned)})
+                                                                 "tiling": tuned, "tail": tail_of(tb)})
     out["qss_vs_asymptotic_mixed_zones_per_s"] = out["qss_mixed"]["zones_per_s"] / mixed_line["zones_per_s"]
     # the learned proposal: records from training zones, training on the GPU,
     # then the batch with the network proposing and the plain test judging
@@ -584,7 +588,7 @@ def other_forms(kn, g, net, zones, dz, stream, flush, mixed_line, args):
     st = tb["stats"]
     kms = _mean(tb["kernel_ms"])
     roof = smem_roofline([(net, st["steps"], st["rejects"])], kms, tb["clocks"], n_sms,
-                         kernel="integrate_kernel")
+                         kernel=kernel_of())
     # the network evaluation on CUDA cores: 2 (64 128 + 128 128 + 128) flops
     # per proposal, one proposal per state reached by an accepted step
     mlp_flops = 2.0 * (64 * 128 + 128 * 128 + 128) * (st["steps"] - zones.n_zones)
@@ -594,7 +598,7 @@ def other_forms(kn, g, net, zones, dz, stream, flush, mixed_line, args):
                              "peak_source": "derived: 128 FP32 FMA lanes/clk/SM x 2 x SMs x sampled clock"}
     out["mixed_learned"] = _form_line(tb, [g], zones.n_zones, roof, {
         "proposals_used": st["proposals_used"], "median_rel_err_vs_tight_oracle": err(), "tiling": tuned,
-        "tail": tail_of(tb, tuned),
+        "tail": tail_of(tb),
         "records": int(feat.shape[0]), "record_gen_s": rec_s, "train_s": train_s,
         "train_kernel_s": train_kernel_s, "train_loss_first_last": [hist[0], hist[-1]]})
     out["learned_vs_plain_mixed_zones_per_s"] = out["mixed_learned"]["zones_per_s"] / mixed_line["zones_per_s"]
@@ -722,7 +726,7 @@ def qss_chain(kn, stream, flush, fp64_peak):
                                  "as the 150-species forms' FP64 counts")
         else:
             roof = smem_roofline([(net, st["steps"], st["rejects"])], kms, tb["clocks"], n_sms,
-                                 qss=method == kn.METHOD_QSS)
+                                 qss=method == kn.METHOD_QSS, kernel=KERNELS[g.launch_info()["kernel"]])
         Y = g.get(stream)["Y"]
         e = [np.median(np.abs(Y[i][m] - tight["Y"][a][m]) / tight["Y"][a][m])
              for a, i in enumerate(pick) for m in [tight["Y"][a] > 1e-10]]
@@ -770,7 +774,7 @@ def uneven_sizes(kn, stream, flush, n_sms, args):
                      "rejects": st["rejects"], "zones_per_s": st["zones_ok"] / (kms / 1e3),
                      "zone_steps_per_s": st["steps"] / (kms / 1e3), "t_end": UNEVEN_T_END[name]}
         parts.append((net, st["steps"], st["rejects"]))
-    roof = smem_roofline(parts, kms, tb["clocks"], n_sms)
+    roof = smem_roofline(parts, kms, tb["clocks"], n_sms, kernel=KERNELS[gs[0].launch_info()["kernel"]])
     line = _form_line(tb, gs, MIXED_ZONES, roof, {"per_network": per, "tiling": tuned})
     line["tail"] = tail_stats(tb["zone_ns"], np.concatenate(steps_all), None)
     for g in gs:
@@ -903,11 +907,12 @@ def main():
         roof = fp64_roofline(update_fp64_flops(net, st["steps"] + st["rejects"]), kms, kn.measure_fp64_peak(stream),
                              "11 FP64 operations per species per attempt (update, conservation sum, test)")
         roof["smem"] = smem_roofline([(net, st["steps"], st["rejects"])], kms, clk, n_sms,
-                                     kernel="integrate_kernel")
+                                     kernel=KERNELS[g.launch_info()["kernel"]])
     else:
         # SM-local bound: shared-memory bandwidth, 32 banks x 4 B per clock per
         # SM at the SM clock sampled during the timed steps
-        roof = smem_roofline([(net, st["steps"], st["rejects"])], kms, clk, n_sms, qss=args.form == "qss_mixed")
+        roof = smem_roofline([(net, st["steps"], st["rejects"])], kms, clk, n_sms, qss=args.form == "qss_mixed",
+                             kernel=KERNELS[g.launch_info()["kernel"]])
     # DRAM traffic of the integrator from the committed ncu capture of this
     # kernel (small case, mixed form), scaled to this launch by zone count
     # (each zone's state is read once per launch); null when the kernel's
@@ -933,7 +938,7 @@ def main():
         roof["dram_gbs"] = traffic / (kms / 1e3) / 1e9
         roof["dram_frac_of_hbm"] = roof["dram_gbs"] / peaks["hbm_gbs"]
         roof["hbm_peak_source"] = f"MEASURED_PEAKS.json hbm_gbs ({src})"
-    groups = zones_in_flight(tb["zone_ns"]) if tuned or (args.tpz and args.tpc) else None
+    groups = zone_slots(g.launch_info())
     dtype = {"mixed": "f32 (float-float state)", "mixed_fp64": "f32 fluxes, f64 update", "fp64": "f64",
              "qss_fp64": "f64", "qss_mixed": "f32 (float-float state)"}[args.form]
     line = {"metric": METRIC, "value": value, "unit": "zone-steps/s", "n_gpus": world, "steps": args.steps,
@@ -945,7 +950,7 @@ def main():
                        "form": args.form, "l2": "flushed between timed steps (256 MB write)",
                        "accepted_steps_per_batch": int(steps_per_batch), "rejects_per_batch": int(st["rejects"]),
                        "zones_ok": int(zones_ok), "parallelism": f"zones sharded, {world} GPU(s)",
-                       "tiling": tuned if tuned else {"threads_per_zone": args.tpz, "threads_per_cta": args.tpc}},
+                       "launch": g.launch_info(), "tuned": tuned},
             "clocks": clk, "e2e": e2e, "gpu_launches": 3 * args.steps, "roofline": roof,
             "tail": tail_stats(tb["zone_ns"], zone_steps, groups),
             "paper_context": ("the paper estimates ~100 150-isotope networks integrated on one Kepler GPU "
