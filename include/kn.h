@@ -423,10 +423,10 @@ kn_status kn_mlp_adam(kn_mlp *mlp, float lr, float beta1, float beta2, float eps
  * Autotuner and measurement helpers (library additions; the paper has none).
  * ------------------------------------------------------------------------- */
 typedef struct {
-    int32_t threads_per_cta;   /* CTA size P */
+    int32_t threads_per_cta;   /* CTA size P (KN_KERNEL_SLOTS trials: see kn_autotune) */
     int32_t threads_per_zone;  /* zone group size G (G == P: CTA-per-zone) */
     double zone_steps_per_s;   /* measured on the trial batch */
-    int32_t candidates;        /* tilings timed */
+    int32_t candidates;        /* launches timed */
     int32_t pad;
 } kn_tiling;
 
@@ -436,17 +436,22 @@ typedef struct {
  * and learned/plain form (a tiling in opts still overrides it).  Candidates:
  * zone groups from one warp (small networks) or the smallest warp multiple
  * covering the species, up to CTA-per-zone, each with the most groups per CTA
- * that fit in shared memory and with fewer.  Each candidate runs once for one
- * step (building its tables), then is timed.  max_steps > 0: two trials, each
- * integrating the longest predicted zones (the head of the work queue, twelve
- * per SM) for at most max_steps accepted steps -- the steady state of a long
- * batch -- and the better one counts.  max_steps == 0: one trial that
- * integrates the whole batch, which also weighs the tail, where the longest
- * zone's per-step latency rather than throughput can set the batch time.  The
- * zone state is saved before and restored after the trials.  *best receives
- * the winner.  Synchronises
- * `stream`.  Errors: KN_ERR_INVALID_ARG, KN_ERR_STATE (no zones), KN_ERR_NOMEM,
- * KN_ERR_CUDA.
+ * that fit in shared memory and with one fewer.  Where the trial runs
+ * KN_KERNEL_SLOTS (kn_get_launch_info: KN_PREC_MIXED without mlp), which takes
+ * only the order of the sums from a tiling, each zone group size (several
+ * networks: each combination of them) is timed once, and threads_per_cta is not
+ * measured: for one network it is the built-in rule's for that group size, as the
+ * calls that run the group kernel all the same take it (records, replay,
+ * kn_probe_step, or a caller who passes it to kn_integrate_noalloc).  Each
+ * candidate runs once for one step (building its tables), then is timed.
+ * max_steps > 0: two trials, each integrating the longest predicted zones (the
+ * head of the work queue, twelve per SM) for at most max_steps accepted steps --
+ * the steady state of a long batch -- and the better one counts.
+ * max_steps == 0: one trial that integrates the whole batch, which also weighs
+ * the tail, where the longest zone's per-step latency rather than throughput can
+ * set the batch time.  The zone state is saved before and restored after the
+ * trials.  *best receives the winner.  Synchronises `stream`.
+ * Errors: KN_ERR_INVALID_ARG, KN_ERR_STATE (no zones), KN_ERR_NOMEM, KN_ERR_CUDA.
  */
 kn_status kn_autotune(kn_network *const *nets, int32_t n_nets, const kn_opts *opts, int64_t max_steps,
                       void *stream, kn_tiling *best);

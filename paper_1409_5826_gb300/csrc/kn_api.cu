@@ -13,6 +13,7 @@
 #include <functional>
 #include <map>
 #include <memory>
+#include <set>
 #include <string>
 #include <thread>
 #include <vector>
@@ -182,6 +183,9 @@ static kn_status device_info(DeviceInfo& d) {
 struct Tiling {
     int G = 0, M = 0, smem_tables = 1, bytes = 0;
 };
+
+// The built-in tiling's groups per CTA in the mixed form, for groups of several warps.
+constexpr int kTargetGroups = 5;
 
 // Smallest zone group for a network: one warp for small networks; otherwise
 // enough threads (a multiple of 32, at least a warp group) that the FP64
@@ -675,7 +679,6 @@ static kn_status prepare_launch(kn_network* const* nets, int n_nets, const kn_op
             const int g0 = o->threads_per_zone ? o->threads_per_zone : base_group(n);
             const int g1 = o->threads_per_zone ? o->threads_per_zone : 512;
             const bool small = g0 == 32 || prec != kPrecMixed;
-            constexpr int kTargetGroups = 5;
             if ((s = build_tables_range(n, prec, g0, g1)) != KN_OK) return s;
             for (int G = g0; G <= g1; G += 32) {
                 Tables* tb;
@@ -1130,12 +1133,18 @@ cudaError_t launch_fp64_peak(double* out, int blocks, int threads, int iters, cu
 }
 
 namespace {
-// Candidate (P, G) tilings for the listed networks.
+// Candidate tilings for the listed networks: CTA size, group size (0: what the CTA size
+// gives each network), and the CTA size of the built-in rule for that group size, which
+// goes with a candidate whose trial the CTA size does not reach (kn_slots.cu).
+struct Candidate {
+    int P, G, P_rule;
+};
 static kn_status tiling_candidates(kn_network* const* nets, int n_nets, int prec, int extras, int budget,
-                                   std::vector<std::pair<int, int>>& out) {
+                                   std::vector<Candidate>& out) {
     kn_status s;
     if (n_nets == 1) {
         kn_network* n = nets[0];
+        const bool small = base_group(n) == 32 || prec != kPrecMixed;
         for (int G = base_group(n); G <= 512; G += 32) {
             Tables* tb;
             if ((s = get_tables(n, prec, G, &tb)) != KN_OK) return s;
@@ -1146,10 +1155,11 @@ static kn_status tiling_candidates(kn_network* const* nets, int n_nets, int prec
                 M = std::min(kMaxGroups, 1024 / G);
                 while (M > 0 && M * gl.bytes > budget) --M;
             }
-            for (int m = M; m >= std::max(1, M - 1); --m) out.push_back({G * m, G});
+            for (int m = M; m >= std::max(1, M - 1); --m)
+                out.push_back({G * m, G, G * (small ? M : std::min(M, kTargetGroups))});
         }
     } else {
-        for (int P = 1024; P >= 128; P -= 64) out.push_back({P, 0});
+        for (int P = 1024; P >= 128; P -= 64) out.push_back({P, 0, P});
     }
     return KN_OK;
 }
@@ -1202,7 +1212,7 @@ kn_status kn_autotune(kn_network* const* nets, int32_t n_nets, const kn_opts* o,
     const int prec = o->precision;
     const bool learn = o->mlp != nullptr;
     const int budget = di.smem_optin - 1024 - 64 - (learn ? kMlpSmemBytes : 0);
-    std::vector<std::pair<int, int>> cands;
+    std::vector<Candidate> cands;
     const int extras = (learn ? kLayoutFeat : 0) | (o->method == KN_METHOD_QSS ? kLayoutQss : 0);
     if ((s = tiling_candidates(nets, n_nets, prec, extras, budget, cands)) != KN_OK) return s;
     // save the zone abundances (the trials integrate in place)
@@ -1231,10 +1241,11 @@ kn_status kn_autotune(kn_network* const* nets, int32_t n_nets, const kn_opts* o,
     };
     for (int p = 0; p < n_nets; ++p) nets[p]->trial_Z = trial_Z;
     kn_tiling win{0, 0, 0.0, 0, 0};
-    for (const auto& c : cands) {
+    std::set<std::vector<int>> orders;  // of the trials in kn_slots.cu
+    for (const Candidate& c : cands) {
         kn_opts t = *o;
-        t.threads_per_cta = c.first;
-        t.threads_per_zone = c.second;
+        t.threads_per_cta = c.P;
+        t.threads_per_zone = c.G;
         t.use_graph = 0;
         // Untimed first run of one step: builds and uploads the candidate's
         // tables (host work that would otherwise sit between the events) and
@@ -1245,6 +1256,13 @@ kn_status kn_autotune(kn_network* const* nets, int32_t n_nets, const kn_opts* o,
             KN_CUDA(cudaMemcpyAsync(nets[p]->Y.p, saved[p]->p, 8 * (size_t)nets[p]->Z * nets[p]->N,
                                     cudaMemcpyDeviceToDevice, st));
         if (kn_integrate_batch(nets, n_nets, &t, st) != KN_OK) continue;  // does not fit: skipped
+        // kn_slots.cu takes the order of the sums alone from a tiling: one trial an order
+        const bool slots = nets[0]->launched.kernel == KN_KERNEL_SLOTS;
+        if (slots) {
+            std::vector<int> order;
+            for (int p = 0; p < n_nets; ++p) order.push_back(nets[p]->launched.threads_per_zone);
+            if (!orders.insert(order).second) continue;
+        }
         t.max_steps = full ? o->max_steps : std::min<int64_t>(o->max_steps, max_steps);
         double rate = 0.0;
         for (int rep = 0; rep < (full ? 1 : 2) && s == KN_OK; ++rep) {
@@ -1270,9 +1288,9 @@ kn_status kn_autotune(kn_network* const* nets, int32_t n_nets, const kn_opts* o,
         win.candidates += 1;
         if (rate > win.zone_steps_per_s) {
             win.zone_steps_per_s = rate;
-            win.threads_per_cta = c.first;
+            win.threads_per_cta = slots ? c.P_rule : c.P;
             // resolve the group size the launch used for each network
-            win.threads_per_zone = c.second;
+            win.threads_per_zone = c.G;
         }
     }
     cudaEventDestroy(e0);

@@ -169,3 +169,28 @@ def test_several_networks_against_the_group_kernel(env, zones, method):
     assert zones != (1, 0, 900, 0) or gs[0].launch_info()["ctas"] == 0
     for g in gs:
         g.close()
+
+
+@pytest.mark.parametrize("net,zones,smallest", [(chain_network, 700, 32), (net150, 300, 160)])
+def test_autotune_times_each_order_once(env, net, zones, smallest):
+    """Trials of the several-zones kernel differ in the order of the sums alone: one each
+    for the group sizes from the smallest to 512 threads, and the CTA size that comes back
+    is the built-in rule's for the group kernel."""
+    torch, kn = env
+    net = net()
+    z = profile_zones(net, zones, base_seed=45, t_end=3e-12)
+    g = kn.Network(net)
+    g.set_zones(z)
+    t = kn.autotune([g], kn.Opts(precision=kn.PREC_MIXED), max_steps=20)
+    G, M = t["threads_per_zone"], t["threads_per_cta"] // t["threads_per_zone"]
+    assert t["candidates"] == (512 - smallest) // 32 + 1
+    assert t["threads_per_cta"] == G * M and M == min(1024 // G, 15 if smallest == 32 else 5)
+    g.set_zones(z)
+    kn.integrate_batch([g], kn.Opts(precision=kn.PREC_MIXED))
+    i = g.launch_info()
+    assert i["kernel"] == kn.KERNEL_SLOTS and i["threads_per_zone"] == G
+    # a form on the group kernel: as many candidates as before, two for most group sizes
+    g.set_zones(z)
+    t = kn.autotune([g], kn.Opts(precision=kn.PREC_MIXED_FP64), max_steps=20)
+    assert t["candidates"] > (512 - smallest) // 32 + 1
+    g.close()
