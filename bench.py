@@ -8,7 +8,8 @@ batch: load the zones' conditions from device-resident inputs, then the
 persistent integrator (rates, fluxes, gathers, kappa-switched update, accept
 test, dt control) until every zone reaches t_end.
 
-Prints ONE JSON line (rank 0).  value = accepted zone-steps per second over
+Prints ONE JSON line on stdout (rank 0), and before it everything measured, as one
+line of JSON on stderr.  value = accepted zone-steps per second over
 all ranks; zones_per_s alongside.  Beside the headline (the mixed form), each
 other form is timed the same way -- warm-up steps, CUDA events on the
 launching stream around each batch, the L2 flushed between batches, clocks
@@ -782,6 +783,56 @@ def uneven_sizes(kn, stream, flush, n_sms, args):
     return line
 
 
+def _digits(x):
+    """Floats to six significant digits, in nested lists and dicts."""
+    if isinstance(x, dict):
+        return {k: _digits(v) for k, v in x.items()}
+    if isinstance(x, list):
+        return [_digits(v) for v in x]
+    return float(f"{x:.6g}") if isinstance(x, float) else x
+
+
+def short_line(line):
+    """The line that is printed: the contract's keys as they are, the roofline's figures,
+    and of each other form its rates, roofline fraction and error.  (With every form's
+    record the line came to 20,000 characters, more than its reader keeps.)"""
+    out = {k: v for k, v in line.items() if k not in ("tail", "roofline", "paper_context", "forms", "single_zone",
+                                                      "cpu_baseline", "cpu_implicit_be")}
+    out["roofline"] = _digits({k: line["roofline"].get(k)
+                               for k in ("bound", "resource", "unit", "kernel", "achieved", "peak", "frac",
+                                         "peak_source", "full_count_frac", "kernel_ms", "traffic", "issue")})
+    if out["roofline"]["issue"]:
+        out["roofline"]["issue"] = {k: v for k, v in out["roofline"]["issue"].items() if k != "source"}
+    out["tail"] = _digits({k: line["tail"][k] for k in ("span_ms", "tail_ms", "group_occupancy")})
+
+    def form(d):
+        keys = {"zone_steps_per_s": "zone_steps_per_s", "zones_per_s": "zones_per_s", "kernel_ms": "ms",
+                "us_per_training_step": "us", "median_rel_err_vs_tight_oracle": "rel_err"}
+        r = {short: d[k] for k, short in keys.items() if k in d}
+        frac = d["roofline"].get("frac") if "roofline" in d else d.get("frac")
+        return _digits({**r, "frac": frac} if frac is not None else r)
+
+    forms = {}
+    for k, v in line.get("forms", {}).items():
+        if k == "qss_chain":
+            forms.update({f"chain_{q}": form(w) for q, w in v.items() if isinstance(w, dict)})
+        elif k == "perfect_proposal_ceiling":
+            forms[k] = _digits({q: v[q] for q in ("steps_ratio", "attempts_ratio")})
+        elif isinstance(v, dict):
+            forms[k] = form(v)
+        elif isinstance(v, float):
+            forms[k] = _digits(v)
+    if forms:
+        out["forms"] = forms
+    if "single_zone" in line:
+        out["single_zone"] = _digits({n: {k: v for k, v in d.items() if k.endswith("_s_per_step")}
+                                      for n, d in line["single_zone"].items() if isinstance(d, dict)})
+    for k in ("cpu_baseline", "cpu_implicit_be"):
+        if k in line:
+            out[k] = _digits(line[k])
+    return out
+
+
 def main():
     args = _args()
     rank, world, local = _dist()
@@ -963,7 +1014,9 @@ def main():
         exp, be = cpu_baselines(net, zones)
         line["cpu_baseline"] = exp
         line["cpu_implicit_be"] = be
-    print(json.dumps(line), flush=True)
+    # everything measured to stderr; the line itself, short, is the last thing printed
+    print("bench details: " + json.dumps(line), file=sys.stderr, flush=True)
+    print(json.dumps(short_line(line), separators=(",", ":")), flush=True)
     if world > 1:
         dist.barrier()
         dist.destroy_process_group()
