@@ -95,9 +95,9 @@ struct GroupLayout {
 // warps; reactions are dealt to them by aligned blocks of 32.  A worker thread
 // loads its offsets once, into registers, so what it can hold is a compile-time
 // capacity.
-constexpr int kMaxSlots = 4;          // zones per group
+constexpr int kMaxSlots = 2;          // zones per group
 constexpr int kSlotThreads = 512;     // threads per CTA (128 registers each)
-constexpr int kSlotCtlBytes = 256;    // a group's scalars
+constexpr int kSlotCtlBytes = 128;    // a group's scalars
 struct SlotCaps {
     int f1, f2, fa;  // blocks of 1-body, 2-body and any reactions per thread
     int ga, gb;      // words (two terms each) of a thread's two gather slices

@@ -122,7 +122,7 @@ constexpr int kPartStride = (kMlpParams + 3) & ~3;
 constexpr int kTileThreads = 512;
 constexpr int LDF = NF + 8, LDN = NH + 8;  // padded row strides (BF16 elements)
 constexpr int kTileSmem = (NF * LDN + NH * LDN + kTileRows * LDF + 4 * kTileRows * LDN) * 2 +
-                          (3 * NH + 3 * kTileRows) * 4;
+                          (3 * NH + 2 * kTileRows) * 4;
 
 template <bool BWD>
 __global__ void __launch_bounds__(kTileThreads, 1)
@@ -140,8 +140,7 @@ mlp_tile(const float* __restrict__ feat, const float* __restrict__ y, int B, con
     float* b1s = (float*)(dZ1s + kTileRows * LDN);
     float* b2s = b1s + NH;
     float* w3s = b2s + NH;
-    float* outs = w3s + NH;                // [rows]
-    float* douts = outs + kTileRows;       // [rows]
+    float* douts = w3s + NH;               // [rows]
     float* errs = douts + kTileRows;       // [rows]
     const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
     const int r0 = blockIdx.x * kTileRows;

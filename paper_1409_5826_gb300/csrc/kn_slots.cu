@@ -31,6 +31,7 @@
 // ms, 100 zones of it (one an SM) 7.2 -> 3.5 ms, 8001 zones of the 16/48 chain to
 // 1e-3 s 32.6 -> 20.5 ms, 1000 of 365/4400 to 3e-11 s 42.5 -> 37.3 ms, 4096 QSS
 // chains to 1e-2 s 56.9 -> 38.5 ms.
+#include <cstddef>
 #include <cstdint>
 
 #include "kn_device.cuh"
@@ -150,18 +151,10 @@ template <int M> __device__ __forceinline__ uint32_t hi16(uint32_t w, uint32_t b
 template <int NZ> __device__ __forceinline__ void ld_zones(uint32_t a, typename Pack<NZ>::T (&v)[Pack<NZ>::n]) {
     zset<NZ>(v, 0, lds<0>(a));
     if constexpr (NZ > 1) zset<NZ>(v, 1, lds<128>(a));
-    if constexpr (NZ > 2) {
-        zset<NZ>(v, 2, lds<256>(a));
-        zset<NZ>(v, 3, lds<384>(a));
-    }
 }
 template <int NZ> __device__ __forceinline__ void st_zones(uint32_t a, const typename Pack<NZ>::T (&v)[Pack<NZ>::n]) {
     sts<0>(a, zget<NZ>(v, 0));
     if constexpr (NZ > 1) sts<128>(a, zget<NZ>(v, 1));
-    if constexpr (NZ > 2) {
-        sts<256>(a, zget<NZ>(v, 2));
-        sts<384>(a, zget<NZ>(v, 3));
-    }
 }
 // byte address of word v (zone 0) of an interleaved array, from its base
 template <int NZ> __device__ __forceinline__ int at(int v) { return (v >> 5) * (128 * NZ) + (v & 31) * 4; }
@@ -196,6 +189,9 @@ struct SlotCtl {
     double lnT0, lnR0;
 };
 static_assert(sizeof(SlotCtl) <= kSlotCtlBytes, "SlotCtl");
+static_assert(offsetof(SlotCtl, h) == 0 && offsetof(SlotCtl, acc) % 8 == 0 &&
+                  offsetof(SlotCtl, done) == offsetof(SlotCtl, acc) + 4,
+              "h is loaded as a pack, acc and done as a pair");
 
 template <bool WARP> struct SlotSync {
     int id, n;
@@ -286,7 +282,7 @@ __device__ __forceinline__ void refresh_rates(const PlanDev& P, const SlotBase& 
     const int n1 = r.cnt & 15, n2 = r.cnt >> 4 & 15, na = r.cnt >> 8 & 15, cs = 4 * Tw, Ks = 4 * NZ * Tw;
     float u[NZ];
 #pragma unroll
-    for (int z = 0; z < NZ; ++z) u[z] = lds(f.ctl + 32 + 4 * z);  // SlotCtl::u
+    for (int z = 0; z < NZ; ++z) u[z] = lds(f.ctl + (int)offsetof(SlotCtl, u) + 4 * z);
     auto rates = [&](PK (&k)[n]) {
         const float cj = lds(c);
         PK k0[n];
@@ -989,12 +985,12 @@ __device__ __forceinline__ void run_workers(const PlanDev& P, const OptsDev& O, 
             gs.sync();
             // ---- (a) for the candidate states, as the accepted zones' next attempts
             // need it, while the control warp decides ----
-            const uint32_t rm = QSS ? 0u : ldu(ctl + 24);  // SlotCtl::rmask
+            const uint32_t rm = QSS ? 0u : ldu(ctl + (int)offsetof(SlotCtl, rmask));
             if (rm) refresh_rates<NZ>(P, g, tid, Tw, res, f, rm);
             flux_pass<NZ>(res, f);
             gs.sync();
             // ---- (b) the gathers, stored for the accepted zones ----
-            const uint2 ad = ldu2(ctl + 16);  // SlotCtl::acc, done
+            const uint2 ad = ldu2(ctl + (int)offsetof(SlotCtl, acc));
             done = ad.y;
 #pragma unroll
             for (int z = 0; z < NZ; ++z)
