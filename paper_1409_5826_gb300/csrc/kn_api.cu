@@ -549,8 +549,8 @@ static float rate_cache_tol(double cmax) {
     return cmax > 0.0 ? (float)(1.4901161193847656e-08 / (cmax * 0.6931471805599453)) : 3.0e38f;
 }
 
-// ex2.approx(x) is 1 for every FP32 |x| <= 2^-26 (all of them tried on an sm_103
-// device); fl(c u) stays below that while |u| <= 2^-27 / c_max.
+// ex2.approx(x) is 1 for every FP32 |x| <= 2^-26 (tests/test_gpu_rate_factor.py tries
+// all of them on the device); fl(c u) stays below that while |u| <= 2^-27 / c_max.
 static float one_tol(double cmax) { return cmax > 0.0 ? (float)(7.450580596923828e-09 / cmax) : 3.0e38f; }
 
 // Which autotuned tiling a call uses: the plain form's, the learned form's or
