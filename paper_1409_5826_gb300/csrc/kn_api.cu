@@ -251,24 +251,26 @@ static kn_status build_slots(kn_network* n, Tables& tb, bool warp, int budget) {
             j.s = KN_ERR_NOMEM;
         }
     };
-    const int first = warp ? kCapWarp : kCapGroup, last = warp ? kCapWarp : kCapWide;
-    std::vector<Job> more;
+    auto build_all = [&](std::vector<Job>& v) {
+        size_t i = 0;
+        while (i < v.size() && tb.banks.empty()) build(v[i++]);  // the first that comes to the search does it
+        side_by_side(v.size() - i, [&, i](size_t k) { build(v[i + k]); });
+    };
+    const int most = warp ? 1 : kMaxSlotGroups;
+    std::vector<Job> wide;
     for (int NZ = 1; NZ <= 2; ++NZ)
-        for (int cap = first; cap <= last; ++cap) {
-            // the largest group first: where it fits, plan_slots takes no later capacities
-            Job j{slot_threads(warp, 1), NZ, cap, {}, {}, false, KN_OK, {}};
-            if (j.T < slot_min_threads(n, warp)) continue;
-            build(j);
-            const bool enough = j.fits && j.st.bytes + slot_layout(n, j.st, j.T, NZ, true).bytes <= budget;
-            jobs.push_back(std::move(j));
-            for (int ng = 2; ng <= (warp ? 1 : kMaxSlotGroups); ++ng)
-                if (slot_threads(warp, ng) >= slot_min_threads(n, warp))
-                    more.push_back({slot_threads(warp, ng), NZ, cap, {}, {}, false, KN_OK, {}});
-            if (enough) break;
-        }
-    if (!tb.banks.empty()) side_by_side(more.size(), [&](size_t i) { build(more[i]); });
-    else for (Job& j : more) build(j);  // none of the first came to the search
-    for (Job& j : more) jobs.push_back(std::move(j));
+        for (int ng = 1; ng <= most; ++ng)
+            if (slot_threads(warp, ng) >= slot_min_threads(n, warp))
+                jobs.push_back({slot_threads(warp, ng), NZ, warp ? kCapWarp : kCapGroup, {}, {}, false, KN_OK, {}});
+    build_all(jobs);
+    // the wide capacities only where plan_slots can come to them
+    for (const Job& j : jobs) {
+        const int ng = kSlotThreads / j.T;
+        if (!warp && !(j.fits && j.st.bytes + ng * slot_layout(n, j.st, j.T, j.NZ, true).bytes <= budget))
+            wide.push_back({j.T, j.NZ, kCapWide, {}, {}, false, KN_OK, {}});
+    }
+    build_all(wide);
+    for (Job& j : wide) jobs.push_back(std::move(j));
     std::vector<unsigned char> all;
     std::vector<size_t> at;
     for (Job& j : jobs) {
@@ -339,11 +341,31 @@ static kn_status plan_slots(kn_network* const* nets, int n_nets, const Tiling* t
                 bytes = std::max(bytes, st.bytes + ng * sl.bytes);
                 threads = std::max(threads, ng * T);
             };
-            for (int cap = warp ? kCapWarp : kCapGroup; cap <= (warp ? kCapWarp : kCapWide) && !fit; ++cap)
-                for (int ng = most; ng >= 1 && !fit; --ng) try_plan(cap, ng);
+            // The wide capacities spill registers: three groups of them are slower than two
+            // others (100 species, 5 to 8 zones an SM: 1.08 times the group kernel's rate
+            // against 1.40 .. 1.50), but two of them faster than one of the others from five
+            // zones an SM on (165 species, 5 to 27: 1.08 .. 1.28 against 0.98 .. 0.85; 180
+            // species 1.23 .. 1.29 against 1.28 .. 0.98).  Below, one is (180 species, 3 and
+            // 4: 1.67 and 1.42 against 1.21 and 1.25).
+            if (warp) {
+                for (int ng = most; ng >= 1 && !fit; --ng) try_plan(kCapWarp, ng);
+            } else {
+                for (int ng = most; ng >= 2 && !fit; --ng) try_plan(kCapGroup, ng);
+                if (!fit && most >= 2 && zps > 4) try_plan(kCapWide, 2);
+                if (!fit) try_plan(kCapGroup, 1);
+                for (int ng = most; ng >= 1 && !fit; --ng) try_plan(kCapWide, ng);
+            }
             all = fit;
         }
         if (!all) continue;
+        // One group of two zones on an SM against the group kernel's four or five zones: its
+        // step has to be that much shorter, which the QSS step, with two flux passes and
+        // gathers, is not (188 to 192 species, five groups: 0.75 to 1.3 times the group
+        // kernel's rate from five zones an SM on, 0.87 at 27; 200 species, four: 1.22 .. 0.93,
+        // 0.94 at 27; Eq. 3's step: 0.96 .. 1.5).
+        const PlanDev& L = lp.plans[0];
+        if (n_nets == 1 && qss && NZ == 2 && L.ng == 1 && L.T > 32 && (tl[0].M >= 5 ? zps > 4 : tl[0].M == 4 && zps > 15))
+            return KN_OK;
         lp.nz = NZ;
         lp.smem_bytes = bytes;
         block = threads;

@@ -194,3 +194,31 @@ def test_autotune_times_each_order_once(env, net, zones, smallest):
     t = kn.autotune([g], kn.Opts(precision=kn.PREC_MIXED_FP64), max_steps=20)
     assert t["candidates"] > (512 - smallest) // 32 + 1
     g.close()
+
+
+# (species, zones per SM, QSS, kernel, zones per group, groups per CTA): above 160 species a
+# CTA holds two groups at most, in the wide capacities from five zones an SM on; where one
+# group fits alone, the QSS update goes back to the group kernel's five (188 species, from
+# five zones an SM on) or four (200 species, from sixteen on)
+@pytest.mark.parametrize("species,per_sm,method,kernel,nz,groups", [
+    (165, 4, 0, 1, 2, 1), (165, 5, 0, 1, 2, 2), (180, 4, 1, 1, 2, 1), (180, 5, 1, 1, 2, 2), (180, 16, 0, 1, 2, 2),
+    (188, 4, 1, 1, 2, 1), (188, 5, 1, 0, 1, 5), (188, 16, 0, 1, 2, 1), (200, 15, 1, 1, 2, 1), (200, 16, 1, 0, 1, 4),
+    (200, 16, 0, 1, 2, 1), (150, 16, 1, 1, 2, 2), (250, 16, 1, 1, 2, 1),
+])
+def test_groups_per_cta_above_160_species(env, species, per_sm, method, kernel, nz, groups):
+    torch, kn = env
+    net = sweep_network(species)
+    Z = per_sm * torch.cuda.get_device_properties(0).multi_processor_count
+    dz = _device(torch, profile_zones(net, Z, base_seed=46, t_end=2e-12))
+    opts = dict(precision=kn.PREC_MIXED, method=method, max_steps=40)
+    g = kn.Network(net)
+    g.set_zones(dz)
+    kn.integrate_batch([g], kn.Opts(**opts))
+    i = g.launch_info()
+    assert (i["kernel"], i["zones_per_group"], i["groups_per_cta"]) == (kernel, nz, groups)
+    a = g.get()
+    G = i["threads_per_zone"]
+    b = _group_kernel(torch, kn, g, dz, kn.Opts(threads_per_zone=G, threads_per_cta=G, **opts))
+    for k in OUT:
+        assert np.array_equal(a[k], b[k]), k
+    g.close()
