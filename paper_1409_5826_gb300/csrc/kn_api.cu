@@ -50,6 +50,7 @@ static kn_status build_tables(kn_network* n, int prec, int Q, Tables& T) {
     if (s != KN_OK) return s;
     T.blob.reset(new DevBuf());
     KN_CUDA(T.blob->upload(blob.data(), blob.size()));
+    KN_CUDA(DevBuf::upload_wait());
     return KN_OK;
 }
 
@@ -111,6 +112,7 @@ static kn_status build_tables_range(kn_network* n, int prec, int G0, int G1) {
         KN_CUDA(j.T.blob->upload(j.blob.data(), j.blob.size()));
         n->tables.emplace(std::make_pair(prec, j.G), std::move(j.T));
     }
+    KN_CUDA(DevBuf::upload_wait());
     return KN_OK;
 }
 
@@ -281,6 +283,7 @@ static kn_status build_slots(kn_network* n, Tables& tb, bool warp, int budget) {
     }
     tb.slot_blob.reset(new DevBuf());
     if (!all.empty()) KN_CUDA(tb.slot_blob->upload(all.data(), all.size()));
+    KN_CUDA(DevBuf::upload_wait());
     for (size_t i = 0; i < jobs.size(); ++i)
         tb.slots[{jobs[i].T, 8 * jobs[i].NZ + jobs[i].cap}] =
             SlotBlob{tb.slot_blob->as<unsigned char>() + at[i], jobs[i].st, jobs[i].fits};
@@ -418,6 +421,7 @@ kn_status kn_create_network(const kn_network_desc* d, kn_network** out) {
     kn_status s = network_host_setup(d, n, r0);
     if (s != KN_OK) return s;
     KN_CUDA(n->rate0.upload(r0.data(), 8 * r0.size()));
+    KN_CUDA(DevBuf::upload_wait());
     KN_CUDA(n->qhead.ensure(64));
     *out = n.release();
     return KN_OK;
@@ -1390,6 +1394,7 @@ kn_status kn_set_binding_energies(kn_network* n, const double* B) {
     for (int i = 0; i < n->N; ++i)
         if (!std::isfinite(B[i])) return fail(KN_ERR_INVALID_ARG, "kn_set_binding_energies: B[%d] not finite", i);
     KN_CUDA(n->bind.upload(B, 8 * (size_t)n->N));
+    KN_CUDA(DevBuf::upload_wait());
     n->has_bind = true;
     return KN_OK;
 }

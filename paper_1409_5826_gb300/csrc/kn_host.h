@@ -41,13 +41,12 @@ struct DevBuf {
     }
     // Grow to b bytes and copy them from pageable host memory.  Such a copy may return
     // with its last part still on the way, ordered before later work on streams that
-    // follow the default stream only; after the wait it is there for every stream.
+    // follow the default stream only; after upload_wait it is there for every stream.
     cudaError_t upload(const void* src, size_t b) {
-        cudaError_t e = ensure(b);
-        if (e == cudaSuccess) e = cudaMemcpy(p, src, b, cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
-        return e;
+        const cudaError_t e = ensure(b);
+        return e == cudaSuccess ? cudaMemcpy(p, src, b, cudaMemcpyHostToDevice) : e;
     }
+    static cudaError_t upload_wait() { return cudaStreamSynchronize(cudaStreamLegacy); }
     template <class T> T* as() const { return (T*)p; }
 };
 
