@@ -150,7 +150,10 @@ typedef struct {
        from the tiling only the order of its sums, which threads_per_zone sets: how
        many zones and threads share an SM then follows from the zone count, with the
        same results bit for bit.  Networks beyond that kernel's capacities run as
-       tiled. */
+       tiled (kn_get_launch_info tells).  The forms with FP64 in the step take from
+       a tiling that is not given here no more groups per CTA than the zones need,
+       and in KN_PREC_FP64 with up to two zones an SM groups of a multiple of 128
+       threads, in the same order of the sums. */
     int32_t threads_per_cta;
     int32_t threads_per_zone;
     int32_t use_graph;     /* 1: capture the launch sequence in a CUDA graph and replay it */
@@ -487,6 +490,9 @@ kn_status kn_measure_fp64_peak(double *tflops, void *stream);
  * kn_integrate_batch or kn_probe_step call with those opts, e.g. at set-up);
  * opts->threads_per_zone must be set (threads_per_cta 0 means one zone group
  * per CTA); use_graph, replay and mlp must be off.
+ * It runs KN_KERNEL_GROUP in every precision, as tiled (the tables of
+ * KN_KERNEL_SLOTS are kn_integrate_batch's, which builds them when it first
+ * launches that kernel); the results are kn_integrate_batch's bit for bit.
  *
  * Its only scratch (work-queue counter and order) is a fixed device array in
  * the library, 256 KB per device: no call allocates device memory.  The

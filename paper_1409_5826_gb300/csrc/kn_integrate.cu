@@ -63,8 +63,8 @@ __device__ __forceinline__ double exp_neg_small(double x, int degree) {
 // W = 2^53 x (1 - x/2).  W is formed in fixed point, 22 fraction bits, with an error
 // of less than 12 of their units (the roundings of x and of 1 - x/2 included: at most
 // 3), and a W within 64 units of a rounding boundary is left to the FP64 operations.
-// (608 zones of 150/1604: 276 ms with the FP64 factors and products in the accept
-// test, 157 ms with this and ratio_approx.)  Products in integers beside the pipe
+// (2048 zones of 150/1604 to 3e-11 s: 276 ms with the FP64 factors and products in the
+// accept test, 157 ms with this and ratio_approx.)  Products in integers beside the pipe
 // (four 32-bit multiplications and some 25 other instructions) gained nothing: the
 // flux pass's latency grew by what the pipe was spared.
 //

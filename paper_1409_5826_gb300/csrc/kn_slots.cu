@@ -15,7 +15,7 @@
 //   * a worker thread keeps its reactions' and gather terms' offsets and its
 //     reactions' cached rates in registers for the launch: no table word is loaded
 //     and no loop counted in a step.  128 registers and 512 threads an SM: with 80
-//     and 768 and tables in shared memory the 4096-zone batch took 739 ms, not 648;
+//     and 768 and tables in shared memory the 4096-zone batch took 14 % longer;
 //   * the zones' scalar state lives in registers of a warp of its own, 32 / NZ
 //     lanes a zone: one pass of the decision's instructions serves all zones, and
 //     its FP64 work runs beside the update; the species' float-float state and
@@ -27,10 +27,13 @@
 // the terms of a piece, the segmented reduction, the butterflies, the warps), so
 // the results are the group kernel's bit for bit, whatever T and NZ.
 //
-// Measured against the group kernel: 4096 zones of 150/1604 to 1e-9 s 818 -> 640
-// ms, 100 zones of it (one an SM) 7.2 -> 3.5 ms, 8001 zones of the 16/48 chain to
-// 1e-3 s 32.6 -> 20.5 ms, 1000 of 365/4400 to 3e-11 s 42.5 -> 37.3 ms, 4096 QSS
-// chains to 1e-2 s 56.9 -> 38.5 ms.
+// Measured against the group kernel: 4096 zones of 150/1604 to 1e-9 s 814 -> 627 ms, 100
+// zones of it (one an SM) 7.2 -> 3.5 ms, 8001 zones of the 16/48 chain to 1e-3 s 32.6 ->
+// 20.5 ms, 1000 of 365/4400 to 1e-10 s 52 -> 41 ms, 4096 QSS chains to 1e-2 s 56.9 -> 38
+// ms.  Where it is not faster plan_slots (kn_api.cu) leaves the call to that kernel, except
+// that it cannot see this: with 4 to 5 zones an SM and four slots the fifth zone follows
+// alone, in a pair's step.  Zones of a spread fill that time (684 of 150/1604 1.5 times the
+// group kernel's rate); zones that all take the same number of steps do not (0.8).
 #include <cstddef>
 #include <cstdint>
 
