@@ -1261,13 +1261,17 @@ __device__ __forceinline__ void run_group(const PlanDev& P, const OptsDev& O, co
     // A home CTA's groups start with zones dealt over the CTAs, then over the groups: the
     // queue's first zones take the most steps, and where the groups of one CTA took them
     // from the queue side by side, that SM finished last (1024 zones of 150/1604 to
-    // 1e-10 s, FP64 update: 192 -> 140 ms; 512 learned zones: 32.8 -> 30.2).
-    if (lane == 0)
-        S.zone = (int)blockIdx.x >= P.cta_begin && (int)blockIdx.x < P.cta_end ? -2 : -1;
+    // 1e-10 s, FP64 update: 192 -> 140 ms; 512 learned zones: 32.8 -> 30.2).  S.zone holds
+    // the place in the queue between zones, so that the step loop keeps nothing of this in
+    // registers: worked out at the top of the loop it cost every mixed-form step 2 to 3 %
+    // (one zone of 150/1604 to 1e-11 s 3.03 -> 3.09 ms, 3.03 like this).
+    if (lane == 0) {
+        const int b = (int)blockIdx.x - P.cta_begin, n = P.cta_end - P.cta_begin;
+        S.zone = b >= 0 && b < n ? gr * n + b : P.dealt + atomicAdd(P.queue_head, 1);
+    }
     for (;;) {
         if (lane == 0) {
-            const int q = S.zone == -2 ? gr * (P.cta_end - P.cta_begin) + (int)blockIdx.x - P.cta_begin
-                                       : P.dealt + atomicAdd(P.queue_head, 1);
+            const int q = S.zone;
             S.zone = q < P.n_zones ? P.order[q] : -1;
             S.valid = 1;
             if (O.zone_ns) S.t_fetch_ns = global_ns();
@@ -1659,6 +1663,7 @@ __device__ __forceinline__ void run_group(const PlanDev& P, const OptsDev& O, co
                 }
             }
         }
+        if (lane == 0) S.zone = P.dealt + atomicAdd(P.queue_head, 1);  // the next one's place in the queue
         gs.sync();
     }
 }
