@@ -44,13 +44,31 @@ const char* last_error() { return g_err.c_str(); }
 
 namespace {
 
-static kn_status build_tables(kn_network* n, int prec, int Q, Tables& T) {
+// Tables built on the host into the network's, all in one allocation and one copy.
+struct TableJob {
+    int G;
     std::vector<unsigned char> blob;
-    kn_status s = build_tables_host(n, prec, Q, blob, T);
-    if (s != KN_OK) return s;
-    T.blob.reset(new DevBuf());
-    KN_CUDA(T.blob->upload(blob.data(), blob.size()));
+    Tables T;
+    kn_status s;
+    std::string msg;
+};
+static kn_status add_tables(kn_network* n, int prec, std::vector<TableJob>& jobs) {
+    std::vector<unsigned char> all;
+    std::vector<size_t> at;
+    for (TableJob& j : jobs) {
+        if (j.s != KN_OK) return fail(j.s, "%s", j.msg.c_str());
+        at.push_back(all.size());
+        all.insert(all.end(), j.blob.begin(), j.blob.end());
+        all.resize((all.size() + 255) / 256 * 256);
+    }
+    std::unique_ptr<DevBuf> mem(new DevBuf());
+    KN_CUDA(mem->upload(all.data(), all.size()));
     KN_CUDA(DevBuf::upload_wait());
+    for (size_t i = 0; i < jobs.size(); ++i) {
+        jobs[i].T.dev = mem->as<unsigned char>() + at[i];
+        n->tables.emplace(std::make_pair(prec, jobs[i].G), std::move(jobs[i].T));
+    }
+    n->table_mem.push_back(std::move(mem));
     return KN_OK;
 }
 
@@ -58,10 +76,11 @@ static kn_status get_tables(kn_network* n, int prec, int Q, Tables** out) {
     auto key = std::make_pair(prec, Q);
     auto it = n->tables.find(key);
     if (it == n->tables.end()) {
-        Tables T;
-        kn_status s = build_tables(n, prec, Q, T);
-        if (s != KN_OK) return s;
-        it = n->tables.emplace(key, std::move(T)).first;
+        std::vector<TableJob> job(1);
+        job[0].G = Q;
+        kn_status s = job[0].s = build_tables_host(n, prec, Q, job[0].blob, job[0].T);
+        if (s != KN_OK || (s = add_tables(n, prec, job)) != KN_OK) return s;
+        it = n->tables.find(key);
     }
     *out = &it->second;
     return KN_OK;
@@ -86,19 +105,12 @@ template <class F> static void side_by_side(size_t count, F f) {
 // The tables of every group size G0, G0 + 32, .. G1, the missing ones built side by
 // side: a default launch looks at up to 12 of them (5 ms each for 150/1604).
 static kn_status build_tables_range(kn_network* n, int prec, int G0, int G1) {
-    struct Job {
-        int G;
-        std::vector<unsigned char> blob;
-        Tables T;
-        kn_status s;
-        std::string msg;
-    };
-    std::vector<Job> jobs;
+    std::vector<TableJob> jobs;
     for (int G = G0; G <= G1; G += 32)
         if (!n->tables.count({prec, G})) jobs.push_back({G, {}, {}, KN_OK, {}});
     if (jobs.size() < 2) return KN_OK;  // get_tables builds it
     side_by_side(jobs.size(), [&](size_t i) {
-        Job& j = jobs[i];
+        TableJob& j = jobs[i];
         try {
             j.s = build_tables_host(n, prec, j.G, j.blob, j.T);
             if (j.s != KN_OK) j.msg = last_error();  // the message is this thread's
@@ -106,14 +118,7 @@ static kn_status build_tables_range(kn_network* n, int prec, int G0, int G1) {
             j.s = KN_ERR_NOMEM;
         }
     });
-    for (Job& j : jobs) {
-        if (j.s != KN_OK) return fail(j.s, "%s", j.msg.c_str());
-        j.T.blob.reset(new DevBuf());
-        KN_CUDA(j.T.blob->upload(j.blob.data(), j.blob.size()));
-        n->tables.emplace(std::make_pair(prec, j.G), std::move(j.T));
-    }
-    KN_CUDA(DevBuf::upload_wait());
-    return KN_OK;
+    return add_tables(n, prec, jobs);
 }
 
 // The FP32-flux forms keep a per-group cache of the current rates (4 R bytes)
@@ -752,7 +757,7 @@ static kn_status prepare_launch(kn_network* const* nets, int n_nets, const kn_op
         if ((s = get_tables(n, prec, t.G, &tb)) != KN_OK) return s;
         const GroupLayout gl = group_layout(n, prec, t.G, extras);
         PlanDev& P = lp.plans[p];
-        P.blob = (const unsigned char*)tb->blob->p;
+        P.blob = tb->dev;
         P.tl = tb->tl;
         P.rate0 = n->rate0.as<const double2>();
         P.R1 = n->R1;
@@ -1089,7 +1094,7 @@ kn_status noalloc_prepare(kn_network* n, const kn_opts* o, int32_t n_zones, cons
     lp.n_plans = 1;
     lp.smem_bytes = bytes;
     PlanDev& Pd = lp.plans[0];
-    Pd.blob = (const unsigned char*)tb.blob->p;
+    Pd.blob = tb.dev;
     Pd.tl = tb.tl;
     Pd.rate0 = n->rate0.as<const double2>();
     Pd.R1 = n->R1;

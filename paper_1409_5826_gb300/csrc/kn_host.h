@@ -68,7 +68,7 @@ struct SlotBlob {
 };
 
 struct Tables {
-    std::unique_ptr<DevBuf> blob;
+    const unsigned char* dev = nullptr;              // in one of kn_network::table_mem
     TableLayout tl{};
     GatherOrder order;                               // mixed form
     std::vector<int> banks;                          // kn_slots.cu: V's values' banks, found on first use
@@ -96,7 +96,8 @@ struct kn_network {
     double cmax = 0;
     kn::DevBuf rate0;                            // double2[R] (ln k0, n), sorted order
     double nbar = 0, rbar = 0;
-    std::map<std::pair<int, int>, kn::Tables> tables;  // (precision, Q) -> device blob
+    std::map<std::pair<int, int>, kn::Tables> tables;  // (precision, Q) -> table
+    std::vector<std::unique_ptr<kn::DevBuf>> table_mem;
     // zone state
     int Z = 0, capZ = 0;
     kn::DevBuf Y, T0, rho0, tau, ts, te, dtt, tout, dtn, steps, rej, props, status, energy;
